@@ -24,9 +24,8 @@
 // words, so a warp reading one crystal down 32 rows hits 32 banks): one
 // shuffle forms a column's differences and one 32 x 32 bit transpose across
 // the warp turns them into bit planes held by lanes in stream order, shared
-// by two or four columns when their widths allow.  The decoder is the same
-// walk backwards (one load of the columns' words, the transpose, the
-// differences summed by an inclusive warp scan).  (One ballot per plane, the
+// by two or four columns when their widths allow.  The decoder puts lanes on
+// crystal columns (see unpack_kernel).  (One ballot per plane, the
 // first form, took 2.7x as long: the integer pipe ran out.  A single pass
 // whose warps found their block's place by decoupled look-back was slower
 // still: with thousands of one-block warps in flight the nearest published
@@ -489,14 +488,121 @@ __global__ void __launch_bounds__(kThreads, 4) pack_write_kernel(const int16_t *
     if (lane == 0) pipe.drain();
 }
 
-__global__ void __launch_bounds__(kThreads) unpack_kernel(const unsigned char *in, long long in_bytes, long long rows,
-                                                          int X, long long nb, int16_t *pool_out, int *err)
+// ------------------------------------------------------------------ decoder
+// Bound by instruction issue and, at the end, by HBM (61% of its rate).  Lanes
+// own crystal columns, two neighbouring ones each (np = ceil(X / 2) lanes a
+// block, nsub = 32 / np blocks side by side), so a column's bit planes become
+// samples inside one lane: seven three-input operations undo the zigzag on the
+// planes, three stages of bit swaps among eight words (48 operations) turn
+// them into 32 signed bytes (word k, byte j = row 8j + k), and one dp4a a row
+// takes its byte and adds it to the running sample.  A row is one 32-bit store
+// of the lane's two samples; whole blocks leave by bulk copy.  With lanes on
+// rows a column took a 32 x 32 transpose and a prefix sum across the warp, 49
+// instructions a column and warp against 12 here: 12.06 M rows x 54 decoded in
+// 1.19 ms, now 0.34 (the call 1275 -> 383 us).
+// Where the columns' words begin is known only by walking their head words, a
+// chain of X shared-memory loads, so a warp stages the payload of up to G = 4
+// consecutive blocks (16-byte asynchronous copies) and G lanes walk them at
+// once; more would cost occupancy (10 KB a warp, 20 warps an SM).  The next
+// group's payload is brought into L2 while this one is decoded (390 -> 383
+// us).  Undoing the zigzag on bytes after the swaps, copying rows out with
+// 16-byte stores and checking every head word in the walk took 502 us.
+// Columns wider than 8 bits (pulses: 2% of the blocks of a dense fill hold
+// one) take the same swaps on planes 8..15 and add plane 16 bit by bit.
+constexpr int kDecWarps = 4;
+constexpr int kDecThreads = 32 * kDecWarps;
+
+// Lanes, blocks and shared memory of one warp, by the crystal count.
+struct DecPlan {
+    int np, nsub, G, cap;  // cap: bytes of staged payload
+    __host__ __device__ explicit DecPlan(int X)
+    {
+        np = (X + 1) / 2;
+        nsub = 32 / np < 16 ? 32 / np : 16;
+        G = nsub >= 4 ? nsub : nsub == 3 ? 6 : 4;
+        // planes of 6.5 bits a column; one block of the widest columns always fits
+        const int want = G * X * 30, least = X * 72;
+        cap = ((want > least ? want : least) + 15) & ~15;
+    }
+    __host__ __device__ size_t pos_at() const { return (size_t)cap + 32; }  // staged words begin at any 4-byte phase
+    __host__ __device__ size_t out_at(int X) const { return (pos_at() + 2 * (size_t)G * X + 15) & ~size_t(15); }
+    __host__ __device__ size_t bytes(int X) const { return out_at(X) + (size_t)nsub * 64 * X; }
+};
+
+// Bit k of byte j of word m -> bit m of byte j of word k (8 x 8 per byte).
+__device__ __forceinline__ void swap_bits8(uint32_t (&p)[8])
 {
-    __shared__ __align__(16) int16_t sm_all[kWarps][kBlockElems];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t a = p[k], b = p[k + 4];
+        p[k] = (a & 0x0f0f0f0fu) | ((b << 4) & 0xf0f0f0f0u);
+        p[k + 4] = ((a >> 4) & 0x0f0f0f0fu) | (b & 0xf0f0f0f0u);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int k = (i & 1) + 4 * (i >> 1);
+        const uint32_t a = p[k], b = p[k + 2];
+        p[k] = (a & 0x33333333u) | ((b << 2) & 0xccccccccu);
+        p[k + 2] = ((a >> 2) & 0x33333333u) | (b & 0xccccccccu);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int k = 2 * i;
+        const uint32_t a = p[k], b = p[k + 1];
+        p[k] = (a & 0x55555555u) | ((b << 1) & 0xaaaaaaaau);
+        p[k + 1] = ((a >> 1) & 0x55555555u) | (b & 0xaaaaaaaau);
+    }
+}
+
+// The differences of a column of width w <= 8 as signed bytes: its zigzag
+// codes' sign plane is plane 0, and bit k of the difference is plane k + 1
+// xor the sign, so seven three-input operations on the planes undo the zigzag
+// of 32 samples.  Words read past the column's planes are masked away.
+__device__ __forceinline__ void column_steps(const uint32_t *h, int w, uint32_t (&p)[8])
+{
+    const uint32_t sign = h[1] & (uint32_t)(-w >> 31);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) p[k] = (h[2 + k] & (uint32_t)((k + 1 - w) >> 31)) ^ sign;
+    p[7] = sign;
+    swap_bits8(p);
+}
+
+// Planes [k0, k0 + 8) of a column as bytes; planes past its width are zero.
+__device__ __forceinline__ void column_bytes(const uint32_t *h, int w, int k0, uint32_t (&p)[8])
+{
+#pragma unroll
+    for (int k = 0; k < 8; ++k) p[k] = k0 + k < w ? h[1 + k0 + k] : 0u;
+    swap_bits8(p);
+}
+
+// One column of any width (<= 17) into every row of the block at out (pitch X).
+__device__ __noinline__ void decode_wide_column(const uint32_t *h, int X, int16_t *out)
+{
+    const int w = (int)(h[0] >> 16);
+    uint32_t lo[8], hi[8];
+    column_bytes(h, w, 0, lo);
+    column_bytes(h, w, 8, hi);
+    const uint32_t top = w > 16 ? h[17] : 0u;
+    int32_t v = (int16_t)(h[0] & 0xffffu);
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+        const int k = r & 7, j = r >> 3;
+        const uint32_t z = ((lo[k] >> (8 * j)) & 0xffu) | (((hi[k] >> (8 * j)) & 0xffu) << 8) | (((top >> r) & 1u) << 16);
+        if (r) v += unzigzag(z);
+        out[r * X] = (int16_t)v;
+    }
+}
+
+template <bool kEven>
+__global__ void __launch_bounds__(kDecThreads, 5) unpack_kernel(const unsigned char *in, long long in_bytes, long long rows,
+                                                             int X, long long nb, int16_t *pool_out, int *err)
+{
+    extern __shared__ __align__(16) unsigned char dsm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int16_t *sm = sm_all[warp];
-    const int P = X;
-    const Transpose transpose(lane);
+    const DecPlan pl(X);
+    unsigned char *base = dsm + warp * pl.bytes(X);
+    uint16_t *pos = reinterpret_cast<uint16_t *>(base + pl.pos_at());  // [G][X] word of each column's head
+    int16_t *out = reinterpret_cast<int16_t *>(base + pl.out_at(X));   // [nsub][32][X]
     const long long head = 16 + 8 * (nb + 1);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const uint32_t *h = reinterpret_cast<const uint32_t *>(in);
@@ -504,94 +610,174 @@ __global__ void __launch_bounds__(kThreads) unpack_kernel(const unsigned char *i
                                                              (unsigned long long)rows)
             atomicOr(err, 1);
     }
-    const unsigned long long *offs = reinterpret_cast<const unsigned long long *>(in + 16);
-    for (long long b = (long long)blockIdx.x * kWarps + warp; b < nb; b += (long long)gridDim.x * kWarps) {
-        if (head > in_bytes) {  // the offsets table itself is cut short
-            if (lane == 0) atomicOr(err, 2);
-            continue;
-        }
-        const unsigned long long off = offs[b];
-        bool bad = off > (unsigned long long)(in_bytes - head) || (off & 3ull);
-        long long pos = head + (long long)(bad ? 0ull : off);  // bytes read so far end at pos
-        for (int x = 0; x < X && !bad;) {
-            // the next 32 words: up to four columns' head words and planes
-            const uint32_t *p = reinterpret_cast<const uint32_t *>(in + pos);
-            const uint32_t q = pos + 4ll * lane + 4 <= in_bytes ? p[lane] : 0u;
-            const uint32_t h0 = __shfl_sync(kFull, q, 0);
-            const int w0 = (int)(h0 >> 16);
-            // four columns of width <= 7 at once: their head words lie at 0, i1, i2, i3
-            const int i1 = 1 + min(w0, 8);
-            const uint32_t h1 = __shfl_sync(kFull, q, i1);
-            const int w1 = (int)(h1 >> 16), i2 = i1 + 1 + min(w1, 8);
-            const uint32_t h2 = __shfl_sync(kFull, q, i2);
-            const int w2 = (int)(h2 >> 16), i3 = i2 + 1 + min(w2, 8);
-            const uint32_t h3 = __shfl_sync(kFull, q, i3);
-            const int w3 = (int)(h3 >> 16), total = i3 + 1 + min(w3, 8);
-            if (x + 3 < X && max(max(w0, w1), max(w2, w3)) <= 7 && pos + 4ll * total <= in_bytes) {
-                // lane 8g + k + 1 takes plane k of column g: the transpose gives lane i
-                // bit k of z_{g,i} at bit 8g + k + 1
-                const int g = lane >> 3, k = lane & 7;
-                const int ig = g == 0 ? 0 : g == 1 ? i1 : g == 2 ? i2 : i3;
-                const int wg = g == 0 ? w0 : g == 1 ? w1 : g == 2 ? w2 : w3;
-                const uint32_t pl = __shfl_sync(kFull, q, (ig + k) & 31);
-                const uint32_t t = transpose(k >= 1 && k <= wg ? pl : 0u);
-                // |difference| <= 64, so 32 of them sum below 2^15: two columns share a scan
-                int32_t d01 = lane ? unzigzag((t >> 1) & 0x7fu) + unzigzag((t >> 9) & 0x7fu) * 65536 : 0;
-                int32_t d23 = lane ? unzigzag((t >> 17) & 0x7fu) + unzigzag((t >> 25) & 0x7fu) * 65536 : 0;
-#pragma unroll
-                for (int s = 1; s < 32; s <<= 1) {
-                    const int32_t y01 = __shfl_up_sync(kFull, d01, s), y23 = __shfl_up_sync(kFull, d23, s);
-                    if (lane >= s) {
-                        d01 += y01;
-                        d23 += y23;
-                    }
-                }
-                const int32_t s0 = (int16_t)(d01 & 0xffff), s2 = (int16_t)(d23 & 0xffff);
-                const int32_t s1 = (d01 - s0) >> 16, s3 = (d23 - s2) >> 16;
-                int16_t *r = sm + lane * P + x;
-                r[0] = (int16_t)((int32_t)(int16_t)(h0 & 0xffffu) + s0);
-                r[1] = (int16_t)((int32_t)(int16_t)(h1 & 0xffffu) + s1);
-                r[2] = (int16_t)((int32_t)(int16_t)(h2 & 0xffffu) + s2);
-                r[3] = (int16_t)((int32_t)(int16_t)(h3 & 0xffffu) + s3);
-                pos += 4ll * total;
-                x += 4;
-                continue;
-            }
-            // one column
-            if (pos + 4 > in_bytes || w0 > 17 || pos + 4ll * (1 + w0) > in_bytes) {
-                bad = true;
-                break;
-            }
-            pos += 4ll * (1 + w0);
-            // lane k + 1 holds plane k: the transpose gives lane i bit k of z_i at bit k + 1
-            const uint32_t z = transpose(lane >= 1 && lane <= w0 ? q : 0u) >> 1;
-            int32_t d = lane ? unzigzag(z) : 0;
-#pragma unroll
-            for (int s = 1; s < 32; s <<= 1) {
-                const int32_t y = __shfl_up_sync(kFull, d, s);
-                if (lane >= s) d += y;
-            }
-            sm[lane * P + x] = (int16_t)((int32_t)(int16_t)(h0 & 0xffffu) + d);
-            ++x;
-        }
-        if (bad) {
-            if (lane == 0) atomicOr(err, 2);
-            continue;
-        }
-        __syncwarp();
-        const long long r0 = 32ll * b;
-        const int nv = (int)min(32ll, rows - r0);
-        int16_t *dst = pool_out + r0 * X;
-        const int n = nv * X;
-        int done = 0;
-        if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) {  // 16-byte vectors where the output allows
-            const int nvec = n >> 3;
-            for (int k = lane; k < nvec; k += 32) reinterpret_cast<int4 *>(dst)[k] = reinterpret_cast<const int4 *>(sm)[k];
-            done = nvec << 3;
-        }
-        for (int e = done + lane; e < n; e += 32) dst[e] = sm[e];
-        __syncwarp();
+    if (head > in_bytes) {  // the offsets table itself is cut short
+        if (threadIdx.x == 0 && nb > 0) atomicOr(err, 2);
+        return;
     }
+    const unsigned long long *offs = reinterpret_cast<const unsigned long long *>(in + 16);
+    const unsigned long long plen = (unsigned long long)(in_bytes - head);  // payload bytes there are
+    const unsigned long long most = 72ull * X;                              // of one block
+    const bool vec_out = (reinterpret_cast<uintptr_t>(pool_out) & 15) == 0;  // then every block is 16-byte aligned
+    const int sub = lane / pl.np, pr = lane - sub * pl.np;
+    const long long step = (long long)gridDim.x * kDecWarps * pl.G;
+    long long b0 = ((long long)blockIdx.x * kDecWarps + warp) * pl.G;
+    // the rows' last bulk copy has read them (the lanes that issued one wait): they may be rewritten
+    auto bulk_read_done = [&] {
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        __syncwarp();
+    };
+    auto offset_of = [&](long long b) { return lane <= pl.G && b + lane <= nb ? offs[b + lane] : ~0ull; };
+    unsigned long long next_off = b0 < nb ? offset_of(b0) : 0ull;
+    for (; b0 < nb; b0 += step) {
+        const int nblk = (int)min((long long)pl.G, nb - b0);
+        const unsigned long long off = next_off;  // of block b0 + lane
+        if (b0 + step < nb) next_off = offset_of(b0 + step);
+        const unsigned long long end = __shfl_down_sync(kFull, off, 1);
+        const bool ok = lane < nblk && off <= plen && !(off & 3ull);
+        // regular: the next offset closes a block of a possible size
+        const bool regular = ok && end <= plen && !(end & 3ull) && end > off && end - off <= most;
+        const unsigned m_ok = __ballot_sync(kFull, ok), m_reg = __ballot_sync(kFull, regular);
+        unsigned alone = 0;  // blocks whose words run past their regular end: staged again by themselves
+        int i = 0;
+        bool bad = lane < nblk && !ok;
+        while (i < nblk || alone) {
+            int g0, n;
+            bool single = false;
+            unsigned long long s0, s1;  // payload bytes staged
+            if (alone) {
+                g0 = __ffs(alone) - 1;
+                alone &= alone - 1u;
+                single = true;
+            } else {
+                g0 = i;
+                if (!((m_ok >> g0) & 1u)) {
+                    ++i;
+                    continue;
+                }
+                single = !((m_reg >> g0) & 1u);
+            }
+            s0 = __shfl_sync(kFull, off, g0);
+            if (single) {
+                n = 1;
+                s1 = min(s0 + most, plen);
+            } else {
+                const unsigned fit = __ballot_sync(kFull, regular && lane >= g0 && end - s0 <= (unsigned long long)pl.cap);
+                n = __ffs(~(fit >> g0)) - 1;
+                s1 = __shfl_sync(kFull, end, g0 + n - 1);
+            }
+            if (g0 == i) i += n;
+            // stage [s0, s1): whole 16-byte units of the stream, then its last words
+            const long long a = head + (long long)s0, e = head + (long long)s1;
+            const long long a16 = a & ~15ll, e16 = min((e + 15) & ~15ll, in_bytes & ~15ll);
+            const uint32_t dst = daq::smem_addr(base);
+            for (long long u = a16 + 16 * lane; u < e16; u += 512)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(u - a16)), "l"(in + u)
+                             : "memory");
+            uint32_t *words = reinterpret_cast<uint32_t *>(base);
+            const long long t0 = max(a16, e16) + 4 * lane;
+            if (t0 + 4 <= e) words[(t0 - a16) >> 2] = *reinterpret_cast<const uint32_t *>(in + t0);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncwarp();
+            if (i >= nblk && !alone && b0 + step < nb) {
+                // the last run of this group: bring the next group's payload into L2 meanwhile
+                const int nn = (int)min((long long)pl.G, nb - b0 - step);
+                const unsigned long long f0 = __shfl_sync(kFull, next_off, 0), f1 = __shfl_sync(kFull, next_off, nn);
+                if (lane == 0 && f0 < f1 && f1 <= plen && f1 - f0 <= most * pl.G) {
+                    const long long q0 = (head + (long long)f0) & ~15ll, q1 = (head + (long long)f1) & ~15ll;
+                    if (q1 > q0)
+                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(in + q0), "r"((uint32_t)(q1 - q0))
+                                     : "memory");
+                }
+            }
+            // walk the head words, one block a lane
+            const int lim = (int)((e - a16) >> 2);  // words staged end here
+            const unsigned long long my_off = __shfl_sync(kFull, off, (g0 + lane) & 31);
+            bool good = false;
+            if (lane < n && lim > 0) {
+                // p only grows, so it ends within the staged words when it
+                // always was (reads past them are held at the last one)
+                int p = (int)((head + (long long)my_off - a16) >> 2), widest = 0;
+                uint16_t *at = pos + lane * X;
+#pragma unroll 6
+                for (int x = 0; x < X; ++x) {
+                    const int q = min(p, lim - 1);
+                    const int w = (int)(words[q] >> 16);
+                    at[x] = (uint16_t)q;
+                    widest = max(widest, w);
+                    p += 1 + w;
+                }
+                good = p <= lim && widest <= 17;
+            }
+            __syncwarp();
+            const unsigned m_good = __ballot_sync(kFull, good);
+            const unsigned m_rest = __ballot_sync(kFull, lane < n) & ~m_good;
+            // staged alone, a block is cut short or has an impossible width;
+            // staged with others it may run past its regular end and is tried again
+            if (single) bad |= m_rest != 0u;
+            else alone |= m_rest << g0;
+            for (int r = 0; r < n; r += pl.nsub) {
+                const int g = r + sub;
+                const bool mine = sub < pl.nsub && g < n && ((m_good >> g) & 1u);
+                const int x0 = 2 * pr;
+                const bool two = mine && x0 + 1 < X;
+                const uint32_t *h0 = words + (mine ? pos[g * X + x0] : 0);
+                const uint32_t *h1 = words + (two ? pos[g * X + x0 + 1] : 0);
+                const uint32_t v0 = mine ? h0[0] : 0u, v1 = two ? h1[0] : 0u;
+                const int w0 = (int)(v0 >> 16), w1 = (int)(v1 >> 16);
+                int16_t *o = out + (sub < pl.nsub ? sub : 0) * 32 * X + x0;
+                if (!__any_sync(kFull, max(w0, w1) > 8)) {
+                    uint32_t p0[8], p1[8];
+                    column_steps(h0, w0, p0);
+                    column_steps(h1, w1, p1);
+                    bulk_read_done();
+                    int32_t a0 = (int32_t)v0, a1 = (int32_t)v1;  // the low halves count
+                    if (mine) {
+#pragma unroll
+                        for (int q = 0; q < 32; ++q) {
+                            const int k = q & 7, j = q >> 3;
+                            if (q) {
+                                a0 = __dp4a((int)p0[k], 1 << (8 * j), a0);
+                                a1 = __dp4a((int)p1[k], 1 << (8 * j), a1);
+                            }
+                            if (kEven) {
+                                *reinterpret_cast<uint32_t *>(o + q * X) = __byte_perm((uint32_t)a0, (uint32_t)a1, 0x5410);
+                            } else {
+                                o[q * X] = (int16_t)a0;
+                                if (two) o[q * X + 1] = (int16_t)a1;
+                            }
+                        }
+                    }
+                } else {
+                    bulk_read_done();
+                    if (mine) decode_wide_column(h0, X, o);
+                    if (two) decode_wide_column(h1, X, o + 1);
+                }
+                __syncwarp();
+                // rows of the good blocks to the pool: a bulk copy per whole block
+                const bool whole = 32 * (b0 + g0 + r + pl.nsub) <= rows;
+                if (vec_out && whole) {
+                    if (pr == 0 && mine) {
+                        daq::fence_proxy_async_smem();
+                        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                                         pool_out + 32 * (b0 + g0 + g) * X),
+                                     "r"(daq::smem_addr(out + sub * 32 * X)), "r"(64 * X)
+                                     : "memory");
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    }
+                } else {
+                    for (int u = 0; u < pl.nsub && r + u < n; ++u) {
+                        if (!((m_good >> (r + u)) & 1u)) continue;
+                        const long long r0 = 32 * (b0 + g0 + r + u);
+                        const int ne = (int)min(32ll, rows - r0) * X;
+                        for (int q = lane; q < ne; q += 32) pool_out[r0 * X + q] = out[u * 32 * X + q];
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        if (bad) atomicOr(err, 2);
+    }
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 // Grid of a pipelined kernel: every CTA resident at once (its warps step
@@ -600,10 +786,11 @@ __global__ void __launch_bounds__(kThreads) unpack_kernel(const unsigned char *i
 // needs (smem_max; a later call must never lower it), and the resident count
 // is found once per (kernel slot, device, n_xtal) and kept.
 constexpr int kGridDevices = 16;
-int g_resident[3][kGridDevices][kMaxX + 1] = {};  // CTAs resident per GPU, 0 = not known yet
-bool g_limit_set[3][kGridDevices] = {};
+int g_resident[5][kGridDevices][kMaxX + 1] = {};  // CTAs resident per GPU, 0 = not known yet
+bool g_limit_set[5][kGridDevices] = {};
 
-template <typename K> int pipelined_grid(int slot, K kernel, int X, size_t smem, size_t smem_max, long long nb)
+template <typename K>
+int pipelined_grid(int slot, K kernel, int X, int threads, size_t smem, size_t smem_max, long long want)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -616,22 +803,12 @@ template <typename K> int pipelined_grid(int slot, K kernel, int X, size_t smem,
                 return 0;
             if (dev < kGridDevices) g_limit_set[slot][dev] = true;
         }
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kThreads, smem) != cudaSuccess || per < 1)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess || per < 1)
             return 0;
         resident = per * sms;
         if (dev < kGridDevices) g_resident[slot][dev][X] = resident;
     }
-    const long long want = (nb + kWarps - 1) / kWarps;
     return (int)std::max<long long>(1, std::min<long long>(want, (long long)resident));
-}
-
-int grid_blocks(long long nb)
-{
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long want = (nb + kWarps - 1) / kWarps;
-    return (int)std::max<long long>(1, std::min<long long>(want, (long long)std::max(sms, 1) * 16));
 }
 
 struct PackWs {
@@ -697,9 +874,10 @@ int daq_pack_pool(const int16_t *pool, int64_t rows, int n_xtal, void *out, int6
     const bool pairs = (n_xtal % 2) == 0;
     const auto write_kernel = pairs ? pack_write_kernel<true> : pack_write_kernel<false>;
     const size_t max_size = kWarps * BlockPipe::bytes(kMaxX, 0), max_write = kWarps * BlockPipe::bytes(kMaxX, kMaxX);
-    const int g_size = nb > 0 ? pipelined_grid(0, pack_size_kernel, n_xtal, smem_size, max_size, nb) : 1;
-    const int g_write = pipelined_grid(pairs ? 1 : 2, write_kernel, n_xtal, smem_write, max_write,
-                                       std::max<long long>(nb, 1));
+    const long long want = (nb + kWarps - 1) / kWarps;
+    const int g_size = nb > 0 ? pipelined_grid(0, pack_size_kernel, n_xtal, kThreads, smem_size, max_size, want) : 1;
+    const int g_write = pipelined_grid(pairs ? 1 : 2, write_kernel, n_xtal, kThreads, smem_write, max_write,
+                                       std::max<long long>(want, 1));
     if (g_size < 1 || g_write < 1) return DAQ_ECUDA;
     if (cudaMemsetAsync(perr, 0, sizeof(int), s) != cudaSuccess) return DAQ_ECUDA;
     if (nb > 0) pack_size_kernel<<<g_size, kThreads, smem_size, s>>>(pool, rows, n_xtal, nb, sizes, widths, perr);
@@ -723,8 +901,15 @@ int daq_unpack_pool(const void *in, int64_t in_bytes, int64_t rows, int n_xtal, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(err, 0, sizeof(int32_t), s) != cudaSuccess) return DAQ_ECUDA;
     const long long nb = (rows + 31) / 32;
-    unpack_kernel<<<grid_blocks(std::max<long long>(nb, 1)), kThreads, 0, s>>>(
-        static_cast<const unsigned char *>(in), in_bytes, rows, n_xtal, nb, pool_out, err);
+    const bool even = (n_xtal % 2) == 0;
+    const auto kernel = even ? unpack_kernel<true> : unpack_kernel<false>;
+    const DecPlan pl(n_xtal);
+    const size_t most = kDecWarps * DecPlan(kMaxX).bytes(kMaxX);
+    const int grid = pipelined_grid(even ? 3 : 4, kernel, n_xtal, kDecThreads, kDecWarps * pl.bytes(n_xtal), most,
+                                    (std::max<long long>(nb, 1) + kDecWarps * pl.G - 1) / (kDecWarps * pl.G));
+    if (grid < 1) return DAQ_ECUDA;
+    kernel<<<grid, kDecThreads, kDecWarps * pl.bytes(n_xtal), s>>>(static_cast<const unsigned char *>(in), in_bytes, rows,
+                                                                    n_xtal, nb, pool_out, err);
     return cudaGetLastError() == cudaSuccess ? DAQ_OK : DAQ_ECUDA;
 }
 

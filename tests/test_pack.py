@@ -134,3 +134,61 @@ def test_short_capacity_and_damaged_streams(env):
         daq.unpack_pool(torch.from_numpy(want[: want.size - 8]).cuda(), 300, 6)
     with pytest.raises(daq.DaqError):                         # header does not match
         daq.unpack_pool(torch.from_numpy(want).cuda(), 299, 6)
+
+
+def _relocated(stream, rows, X, kind, rng):
+    """A stream that decodes to the same rows with its blocks' payloads in
+    another place: in reverse order, with gaps between them, or with every
+    offset but a block's own made useless as the end of the block before it."""
+    nb = -(-rows // 32)
+    head = 16 + 8 * (nb + 1)
+    offs = stream[16:head].view("<u8").astype(np.int64)
+    blocks = [stream[head + offs[b]: head + offs[b + 1]] for b in range(nb)]
+    out, at = [], np.zeros(nb + 1, np.int64)
+    order = range(nb - 1, -1, -1) if kind == "reversed" else range(nb)
+    pos = 0
+    for b in order:
+        if kind == "gaps":
+            out.append(rng.integers(0, 256, 4 * int(rng.integers(0, 40)), dtype=np.uint8))
+            pos += out[-1].size
+        at[b] = pos
+        out.append(blocks[b])
+        pos += blocks[b].size
+    at[nb] = pos
+    if kind == "shared":              # two equal blocks kept once: the next offset lies before the block's end
+        for b in range(1, nb):
+            if np.array_equal(blocks[b], blocks[b - 1]):
+                at[b] = at[b - 1]
+    payload = np.concatenate(out)
+    return np.concatenate([stream[:16], at.astype("<u8").view(np.uint8), payload])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("X", [1, 9, 16, 20, 31, 33, 54, 64])
+@pytest.mark.parametrize("kind", ["plain", "reversed", "gaps", "shared"])
+def test_decoder_follows_any_valid_offsets(env, X, kind):
+    """Crystal counts that put several blocks side by side in a warp, ragged
+    last blocks, narrow and wide columns in one block, and offset tables that a
+    decoder must follow although the blocks do not lie back to back."""
+    torch, daq, oracle = env["torch"], env["daq"], env["oracle"]
+    rng = np.random.default_rng(31 * X + len(kind))
+    rows = 32 * 41 + 13
+    pool = 1800 + np.cumsum(rng.integers(-5, 6, size=(rows, X)), axis=0)
+    wide = rng.integers(0, rows, 40)
+    pool[wide, rng.integers(0, X, 40)] += rng.integers(-30000, 30000, 40)
+    if kind == "shared":
+        pool[64:96] = pool[32:64]
+        pool[96:128] = pool[32:64]
+    pool = pool.astype(np.int16)
+    stream = oracle.pack(pool)
+    if kind != "plain":
+        stream = _relocated(stream, rows, X, kind, rng)
+    assert np.array_equal(oracle.unpack(stream, rows, X), pool)
+    got = daq.unpack_pool(torch.from_numpy(stream).cuda(), rows, X)
+    assert np.array_equal(got.cpu().numpy(), pool)
+    bad = stream.copy()               # a width no encoder writes, in the last block
+    nb = -(-rows // 32)
+    off = int(bad[16 + 8 * (nb - 1): 24 + 8 * (nb - 1)].view("<u8")[0])
+    bad[16 + 8 * (nb + 1) + off + 2] = 18
+    with pytest.raises(daq.DaqError):
+        daq.unpack_pool(torch.from_numpy(bad).cuda(), rows, X)
