@@ -245,7 +245,8 @@ int64_t daq_q_bins(int64_t n_samples, int32_t decim);
  * Process n_fills fills of n_calo calorimeters in one launch sequence.
  *   samples      device int16[n_fills][n_calo][n_xtal][n_samples] (row pitch
  *                n_samples; 12-bit ADC values in 16-bit words, Sec. 3); the
- *                fast path wants 16-byte aligned rows (n_samples % 8 == 0).
+ *                fast path wants 16-byte aligned rows (n_samples % 8 == 0);
+ *                other pitches cost the two-pass form about 1.7x a sample.
  *   n_xtal       crystals per calorimeter, 1..64 (the experiment has 54, Sec. 3).
  *   qhist_inout  device int64 Q histograms (layout: see daq_q_bins); B_D[k] =
  *                sum of S over samples [kD, min(kD + D, len)) is ADDED to bin k

@@ -48,6 +48,7 @@
 #include "daq_twopass.cuh"
 #include "daq_stream.cuh"
 #include "daq_park.cuh"
+#include "daq_launch.cuh"
 
 namespace daq {
 
@@ -716,18 +717,6 @@ constexpr int kSmemPerBlockReserved = 1024;    // reserved by the system for eac
 constexpr int64_t kFusedLagTiles = 1024;
 constexpr int64_t kFusedMinLag = 2 * kCountThreads;
 
-struct Plan {
-    int tw, hl, hr, ew, rs, boxw, nbox, box_stride, slot_bytes, need_sarr, mode;
-    int halo_free;  // two-pass form: the count pass loads the tile proper only
-    int boxw_b, nbox_b, box_stride_b, slot_bytes_b, rs_b;  // compact pass (two-pass mode)
-    size_t smem, smem_b;                                   // tile (or count) kernel, compact kernel
-    int str_meta, str_stages;                              // streaming / single-read forms: tile records, row stages per CTA
-    int pk_slots, pk_cols;                                 // single-read form: park slots, Tensor Memory columns per slot
-    int count_ns;                                          // two-pass form: tile slots of the count kernel (2 or 3)
-    int64_t max_tiles;
-    int64_t ws_tiles;  // tiles the workspace is laid out for: also covers the two-pass plan a call may fall back to
-};
-
 // Box geometry of `width` samples for the compact pass: nbox boxes of boxw <=
 // 248 samples, boxw a multiple of 8.  The compact pass reads along rows, so
 // any row pitch is conflict-free; boxes that split the tile exactly read no
@@ -750,7 +739,7 @@ static size_t count_smem_bytes(int tw, int slot_bytes, int need_sarr)
 static size_t compact_smem_bytes(int tw, int X, int slot_bytes_b)
 {
     size_t b = (size_t)slot_bytes_b + (size_t)(((tw * 2 * X + 32) + 15) & ~15) + (size_t)(tw / 32) * 4 * 6;
-    b += 16 + sizeof(TileInfo) + 2 * sizeof(Agg) + 8 + 8 * (kPlanSmem + 1) + 4 * kPlanSmem + 32;
+    b += 16 + 3 * sizeof(TileInfo) + 2 * sizeof(Agg) + 8 + 8 * (kPlanSmem + 1) + 4 * kPlanSmem + 32;
     return (b + 127) & ~size_t(127);
 }
 
@@ -841,6 +830,27 @@ static void plan_geometry(Plan *pl, int tw, int pre, int post, int X, bool halo_
             pl->smem_b = 0;
         }
     }
+}
+
+// The two-pass plan's slots for row copies (row_load): one box of every column,
+// rows 2 width + 16 bytes apart.  Tile width and workspace stay as planned.
+// False where the wider slots do not fit: the call keeps plain loads.
+static bool rows_geometry(Plan *pl, int X)
+{
+    Plan r = *pl;
+    r.nbox = r.nbox_b = 1;
+    r.boxw = r.ew;
+    r.rs = 2 * r.ew + 16;
+    r.box_stride = r.slot_bytes = (X * r.rs + 127) & ~127;
+    r.boxw_b = r.tw;
+    r.rs_b = 2 * r.tw + 16;
+    r.box_stride_b = r.slot_bytes_b = (X * r.rs_b + 127) & ~127;
+    r.smem = !r.halo_free && r.count_ns == 3 ? CountSmemT<3>::total(r.slot_bytes, r.tw, r.need_sarr)
+                                             : CountSmemT<2>::total(r.slot_bytes, r.tw, r.need_sarr);
+    r.smem_b = compact_smem_bytes(r.tw, X, r.slot_bytes_b);
+    if (r.smem > (size_t)kSmemBudget || r.smem_b > (size_t)kSmemBudget) return false;
+    *pl = r;
+    return true;
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link).
@@ -979,20 +989,6 @@ static int make_plan(int n_calo, int n_xtal, int64_t n_samples, int n_fills, con
     return DAQ_OK;
 }
 
-template <typename K> static cudaError_t ensure_smem(K kernel, size_t bytes, size_t *configured)
-{
-    static std::mutex mu;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    std::lock_guard<std::mutex> g(mu);
-    if (dev >= 0 && dev < 64 && configured[dev] < bytes) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        configured[dev] = bytes;
-    }
-    return cudaSuccess;
-}
-
 template <int TW> static cudaError_t launch_plain(const KArgs &a, const Plan &pl, int grid, cudaStream_t s)
 {
     static size_t configured[64] = {0};
@@ -1018,92 +1014,6 @@ template <int TW> static cudaError_t launch_pipe(const KArgs &a, const Plan &pl,
     if (e != cudaSuccess) return e;
     daq_pipe_kernel<TW><<<grid, kPipeThreads, pl.smem, s>>>(a);
     return cudaGetLastError();
-}
-
-// Launch with programmatic stream serialization: the kernel may be scheduled
-// while the previous kernel of the stream drains; it waits for it in-kernel
-// (pdl_wait) before reading its outputs.
-template <typename K>
-static cudaError_t launch_pdl(K kernel, int grid, int block, size_t smem, cudaStream_t s, const KArgs &a)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return cudaErrorUnknown;
-    cfg.attrs = attr;
-    cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
-}
-
-// The count kernel for NS slots, halo-free or not, grids from occupancy when
-// grid <= 0.
-template <int TW, int NS, bool HF>
-static cudaError_t launch_count(const KArgs &a, const Plan &pl, int grid, int sms, int64_t tiles, cudaStream_t s)
-{
-    static size_t conf[64] = {0};
-    cudaError_t e = ensure_smem(daq_count_kernel<TW, NS, HF>, pl.smem, conf);
-    if (e != cudaSuccess) return e;
-    if (grid <= 0) {
-        int per = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, daq_count_kernel<TW, NS, HF>, count_threads<NS>(), pl.smem);
-        if (e != cudaSuccess) return e;
-        if (per < 1) return cudaErrorInvalidConfiguration;
-        grid = per * sms;
-    }
-    grid = (int)std::min<int64_t>(grid, tiles);
-    return launch_pdl(daq_count_kernel<TW, NS, HF>, grid, count_threads<NS>(), pl.smem, s, a);
-}
-
-// The compact kernel (DAQ_SPARSE: the form that passes over tiles without a
-// marked sample), grids from occupancy when grid <= 0.
-template <int TW, bool kSparse>
-static cudaError_t launch_compact(const KArgs &a, const Plan &pl, int grid, int sms, int64_t tiles, cudaStream_t s)
-{
-    static size_t conf[64] = {0};
-    cudaError_t e = ensure_smem(daq_compact_kernel<TW, kSparse>, pl.smem_b, conf);
-    if (e != cudaSuccess) return e;
-    if (grid <= 0) {
-        int per = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, daq_compact_kernel<TW, kSparse>, 256, pl.smem_b);
-        if (e != cudaSuccess) return e;
-        if (per < 1) return cudaErrorInvalidConfiguration;
-        grid = per * sms;
-    }
-    grid = (int)std::min<int64_t>(grid, tiles);
-    return launch_pdl(daq_compact_kernel<TW, kSparse>, grid, 256, pl.smem_b, s, a);
-}
-
-// Count pass, scan, compact pass.  Events (optional): [2] after the count
-// kernel, [3] after the scan, [4] after the compact kernel.
-template <int TW>
-static cudaError_t launch_twopass(const KArgs &a, const Plan &pl, int grid, int sms, bool skip_isl,
-                                  cudaEvent_t const *ev, cudaStream_t s)
-{
-    cudaError_t e = cudaSuccess;
-    const int64_t tiles = std::max<int64_t>(1, pl.max_tiles);
-    e = pl.halo_free             ? launch_count<TW, 2, true>(a, pl, grid, sms, tiles, s)
-        : pl.count_ns == 3       ? launch_count<TW, 3, false>(a, pl, grid, sms, tiles, s)
-                                 : launch_count<TW, 2, false>(a, pl, grid, sms, tiles, s);
-    if (e != cudaSuccess) return e;
-    if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
-    const int scan_blocks = (int)((tiles + kScanChunk - 1) / kScanChunk);
-    e = pl.halo_free ? launch_pdl(daq_scan_kernel<TW, true>, scan_blocks, kScanThreads, 0, s, a)
-                     : launch_pdl(daq_scan_kernel<TW, false>, scan_blocks, kScanThreads, 0, s, a);
-    if (e != cudaSuccess) return e;
-    if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return e;
-    if (!skip_isl) {
-        e = (a.flags & DAQ_SPARSE) ? launch_compact<TW, true>(a, pl, grid, sms, tiles, s)
-                                   : launch_compact<TW, false>(a, pl, grid, sms, tiles, s);
-        if (e != cudaSuccess) return e;
-    }
-    if (ev && (e = cudaEventRecord(ev[4], s)) != cudaSuccess) return e;
-    return cudaSuccess;
 }
 
 // Streaming single-pass form: one persistent CTA per SM (at most one per tile).
@@ -1221,6 +1131,7 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     KArgs a;
     std::memset(&a, 0, sizeof(a));
     a.samples = samples;
+    a.samples_end = samples ? samples + total : nullptr;
     a.n_calo = n_calo;
     a.n_xtal = n_xtal;
     a.n_fills = n_fills;
@@ -1243,20 +1154,23 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     a.wait_ns = p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs;
     a.fill_len = p.fill_len;
     a.flags = p.flags;
-    a.hl = pl.hl;
-    a.hr = pl.hr;
-    a.ew = pl.ew;
-    a.rs = pl.rs;
-    a.boxw = pl.boxw;
-    a.nbox = pl.nbox;
-    a.box_stride = pl.box_stride;
-    a.slot_bytes = pl.slot_bytes;
-    a.boxw_b = pl.boxw_b;
-    a.nbox_b = pl.nbox_b;
-    a.box_stride_b = pl.box_stride_b;
-    a.slot_bytes_b = pl.slot_bytes_b;
-    a.rs_b = pl.rs_b;
-    a.mode = pl.mode;
+    auto geometry = [&] {
+        a.hl = pl.hl;
+        a.hr = pl.hr;
+        a.ew = pl.ew;
+        a.rs = pl.rs;
+        a.boxw = pl.boxw;
+        a.nbox = pl.nbox;
+        a.box_stride = pl.box_stride;
+        a.slot_bytes = pl.slot_bytes;
+        a.boxw_b = pl.boxw_b;
+        a.nbox_b = pl.nbox_b;
+        a.box_stride_b = pl.box_stride_b;
+        a.slot_bytes_b = pl.slot_bytes_b;
+        a.rs_b = pl.rs_b;
+        a.mode = pl.mode;
+    };
+    geometry();
     a.srow = stage_row_bytes(n_xtal);
     a.wpr = n_xtal / 2;
     a.wpr_mul = a.wpr > 0 ? (1ull << 32) / (unsigned long long)a.wpr + 1 : 0ull;
@@ -1284,25 +1198,16 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
         q.grid = 0;
         rc = make_plan(n_calo, n_xtal, n_samples, n_fills, &q, &pl);
         if (rc) return rc;
-        a.hl = pl.hl;
-        a.hr = pl.hr;
-        a.ew = pl.ew;
-        a.rs = pl.rs;
-        a.boxw = pl.boxw;
-        a.nbox = pl.nbox;
-        a.box_stride = pl.box_stride;
-        a.slot_bytes = pl.slot_bytes;
-        a.boxw_b = pl.boxw_b;
-        a.nbox_b = pl.nbox_b;
-        a.box_stride_b = pl.box_stride_b;
-        a.slot_bytes_b = pl.slot_bytes_b;
-        a.rs_b = pl.rs_b;
-        a.mode = pl.mode;
+        geometry();
         if (total > 0 && n_samples % 8 == 0 && (reinterpret_cast<uintptr_t>(samples) & 15) == 0)
             a.use_tma = encode_tensor_map(&a.tmap, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples, pl.boxw,
                                           n_xtal) &&
                         encode_tensor_map(&a.tmap_b, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples,
                                           pl.boxw_b, n_xtal);
+    }
+    if (pl.mode == kModeTwoPass && !a.use_tma && total > 0 && rows_geometry(&pl, n_xtal)) {
+        a.use_tma = kLoadRows;
+        geometry();
     }
     a.need_sarr = pl.need_sarr;
     a.halo_free = pl.halo_free;
@@ -1369,12 +1274,8 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
         default: e = launch_fused<448>(a, pl, di.sms, ev, s); break;
         }
     } else if (pl.mode == kModeTwoPass) {
-        switch (pl.tw) {
-        case 128: e = launch_twopass<128>(a, pl, p.grid, di.sms, skip_isl, ev, s); break;
-        case 224: e = launch_twopass<224>(a, pl, p.grid, di.sms, skip_isl, ev, s); break;
-        case 384: e = launch_twopass<384>(a, pl, p.grid, di.sms, skip_isl, ev, s); break;
-        default: e = launch_twopass<448>(a, pl, p.grid, di.sms, skip_isl, ev, s); break;
-        }
+        e = a.use_tma == kLoadRows ? launch_twopass_rows(a, pl, p.grid, di.sms, skip_isl, ev, s)
+                                   : launch_twopass_any<false>(a, pl, p.grid, di.sms, skip_isl, ev, s);
     } else if (pl.mode == kModePipelined) {
         int grid = p.grid > 0 ? p.grid : di.sms;
         grid = (int)std::min<int64_t>(grid, tiles_cap);

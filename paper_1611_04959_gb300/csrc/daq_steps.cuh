@@ -23,6 +23,9 @@ constexpr uint64_t kWaitLimitNs = 4000000000ull;  // bounded device waits (4 s)
 constexpr int kMaxTileWords = 14;                 // marks words of the widest two-pass tile (448 samples)
 // kernels a call may use (daq_params.grid picks one)
 enum : int32_t { kModeTwoPass = 0, kModePlain = 1, kModePipelined = 2, kModeFused = 3, kModeStream = 4, kModePark = 5 };
+// daq_params-independent choice of the tile loads: element by element, tensor
+// boxes, or (two-pass form, rows that share no 16-byte alignment) row by row
+enum : int32_t { kLoadPlain = 0, kLoadBoxes = 1, kLoadRows = 2 };
 constexpr int kMaxXtal = 64;
 constexpr int kMaxExtBits = 1024;  // tile + halos: one warp of 32-bit words
 
@@ -98,6 +101,7 @@ struct KArgs {
     CUtensorMap tmap_b;  // the same tensor, boxes of the compact pass (tile proper only)
     CUtensorMap tmap_c;  // the same tensor, 64-sample boxes (the streaming form's compaction steps)
     const int16_t *samples;
+    const int16_t *samples_end;  // one past the last sample of the call
     int32_t n_calo, n_xtal, n_fills;
     int64_t n_samples;  // row pitch
     int32_t threshold, pre, post, ped_samples;
@@ -111,7 +115,7 @@ struct KArgs {
     int32_t hl, hr, ew, rs;  // halo left/right, extended width, smem row pitch (bytes) = 2 boxw
     int32_t boxw, nbox, box_stride, slot_bytes;
     int32_t boxw_b, nbox_b, box_stride_b, slot_bytes_b, rs_b;  // compact pass: tile proper only
-    int32_t use_tma;
+    int32_t use_tma;  // how tiles are loaded: kLoad*
     int32_t mode;
     // two-pass form: the count pass loads the tile proper only (hl = hr = 0)
     // and stores internal marks and crossings; the scan completes the marks
@@ -261,6 +265,72 @@ __device__ __forceinline__ void plain_tile_load(const KArgs &a, const TileInfo &
     }
 }
 
+// Rows whose starts share no 16-byte alignment (n_samples not a multiple of 8,
+// or an input that starts between 16-byte boundaries).  A tile's columns [e0,
+// e0 + width) of a crystal row are copied as the 16-byte units that hold them
+// (asynchronous copies, 512 bytes of a row a warp instruction), so that sample e
+// lies at byte row_phase + 2 (e - e0) of the row's slot (pitch 2 width + 16):
+// the row keeps the byte phase that it has in global memory, and the readers
+// shift a word where that phase is odd in samples.  What else a row's first and
+// last unit hold belongs to its neighbours and is masked like any column outside
+// [0, len).
+// 24 x 54 x 100,003 samples, count + compact kernel: 857 + 829 us with one
+// 2-byte load per sample and a division to find its place, 94 + 121 with one
+// bulk copy per row (54 small bulk copies a tile, about 50 ns each, bound the
+// copy unit), 78 + 101 so.
+__device__ __forceinline__ uint32_t row_phase0(const KArgs &a, long long cf, long long e0)
+{
+    return (uint32_t)(reinterpret_cast<uintptr_t>(a.samples) + 2 * (uintptr_t)(cf * a.n_xtal * a.n_samples + e0)) & 15u;
+}
+
+// One warp: start the copies of columns [e0 + c0, e0 + c1), cut to [0, len), of
+// the tile's rows x0, x0 + dx, ...  No unit that reaches outside the input is
+// copied: its samples, at the input's two ends, are stored one by one.
+__device__ __forceinline__ void row_load(const KArgs &a, const TileInfo &T, unsigned char *slot, int rs, long long e0,
+                                         int c0, int c1, int x0, int dx, int lane)
+{
+    const long long cf = (long long)T.f * a.n_calo + T.c;
+    const uintptr_t in0 = reinterpret_cast<uintptr_t>(a.samples), in1 = reinterpret_cast<uintptr_t>(a.samples_end);
+    long long lo = e0 + c0, hi = e0 + c1;
+    if (lo < 0) lo = 0;
+    if (hi > T.len) hi = T.len;
+    if (lo >= hi) return;
+    const uintptr_t first = in0 + 2 * (uintptr_t)(cf * a.n_xtal * a.n_samples);  // row 0
+    const uintptr_t last = first + 2 * (uintptr_t)((a.n_xtal - 1) * a.n_samples);
+    uintptr_t from = first + 2 * (uintptr_t)((long long)x0 * a.n_samples + lo);  // first byte of row x0
+    const uintptr_t step = 2 * (uintptr_t)((long long)dx * a.n_samples);
+    const uint32_t skip = 2u * (uint32_t)(lo - e0), len = 2u * (uint32_t)(hi - lo);
+    const uint32_t slot_s = smem_addr(slot);
+    const bool inside = ((first + 2 * (uintptr_t)lo) & ~uintptr_t(15)) >= in0 &&
+                        ((last + 2 * (uintptr_t)hi + 15) & ~uintptr_t(15)) <= in1;
+    for (int x = x0; x < a.n_xtal; x += dx, from += step) {
+        const uint32_t ph = ((uint32_t)from - skip) & 15u;  // of column e0
+        const uint32_t units = (((uint32_t)from & 15u) + len + 15u) >> 4;
+        const uintptr_t src = from & ~uintptr_t(15);
+        const uint32_t dst = (uint32_t)(x * rs) + ((ph + skip) & ~15u);  // in the slot
+        if (inside) {
+            for (uint32_t u = lane; u < units; u += 32)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot_s + dst + 16 * u), "l"(src + 16 * u)
+                             : "memory");
+        } else {
+            for (uint32_t u = lane; u < units; u += 32) {
+                const uintptr_t g = src + 16 * u;
+                if (g >= in0 && g + 16 <= in1)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot_s + dst + 16 * u), "l"(g) : "memory");
+                else
+                    for (uintptr_t b = max(g, in0); b < min(g + 16, in1); b += 2)
+                        *reinterpret_cast<int16_t *>(slot + dst + 16 * u + (b - g)) = *reinterpret_cast<const int16_t *>(b);
+            }
+        }
+    }
+}
+// Arrive on `bar` once this thread's copies so far have landed.
+__device__ __forceinline__ void row_load_arrive(uint64_t *bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void row_load_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // --------------------------------------------------------------------------- crystal sum + threshold
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
 {
@@ -281,6 +351,53 @@ __device__ __forceinline__ unsigned long long spread_bits(uint32_t x)
     return v;
 }
 
+// Crystal sums of columns c = 64 it + 2 lane, c + 1 of a tile loaded row by row
+// (every lane of the warp).  The word a lane reads from a row holds its two
+// samples where the row's phase is even in samples, else samples c - 1 and c.
+// The phase's parity is the same for every second row, so crystals of even and
+// of odd index are summed apart as they lie (the inner loop is that of aligned
+// rows), and a sum that lies odd is shifted by a sample once: its low half
+// comes from the next lane, the last lane's from one more word a row, which the
+// lanes read one row each.
+__device__ __forceinline__ void sum_rows(const KArgs &a, const TileInfo &T, uint32_t slot_s, int it, int lane, int &s0,
+                                         int &s1)
+{
+    const int X = a.n_xtal;
+    const int c = 64 * it + 2 * lane;
+    const uint32_t dph = 2u * (uint32_t)a.n_samples;
+    const uint32_t ph0 = row_phase0(a, (long long)T.f * a.n_calo + T.c, T.t0 - a.hl);
+    int lo[2] = {0, 0}, hi[2] = {0, 0};
+    if (c <= a.ew) {  // column ew too: its word may hold sample ew - 1
+        const uint32_t base = slot_s + 2 * c;
+#pragma unroll 9
+        for (int x = 0; x < X; x += 2) {
+            const uint32_t pa = (ph0 + x * dph) & 12u, pb = (ph0 + (x + 1) * dph) & 12u;
+            const uint32_t w0 = lds_u32(base + (uint32_t)(x * a.rs) + pa);
+            const uint32_t w1 = x + 1 < X ? lds_u32(base + (uint32_t)((x + 1) * a.rs) + pb) : 0u;
+            lo[0] = __dp2a_lo((int)w0, 0x0001, lo[0]);
+            hi[0] = __dp2a_lo((int)w0, 0x0100, hi[0]);
+            lo[1] = __dp2a_lo((int)w1, 0x0001, lo[1]);
+            hi[1] = __dp2a_lo((int)w1, 0x0100, hi[1]);
+        }
+    }
+    s0 = s1 = 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        if (!((ph0 + i * dph) & 2u)) {
+            s0 += lo[i];
+            s1 += hi[i];
+            continue;
+        }
+        const int x = 2 * lane + i;
+        int next = __shfl_down_sync(kFull, lo[i], 1), v = 0;
+        if (x < X && 64 * it + 64 <= a.ew)
+            v = (int16_t)(lds_u32(slot_s + 2 * (64 * it + 64) + (uint32_t)(x * a.rs) + ((ph0 + x * dph) & 12u)) & 0xffffu);
+        const int last = __reduce_add_sync(kFull, v);
+        s0 += hi[i];
+        s1 += lane == 31 ? last : next;
+    }
+}
+
 // One warp step of the sum pass over 64 extended columns [64 it, 64 it + 64):
 // lane L owns the two samples of columns c = 64 it + 2L, c + 1, reads their
 // word from every crystal row (conflict-free 4-byte loads) and
@@ -291,6 +408,8 @@ __device__ __forceinline__ unsigned long long spread_bits(uint32_t x)
 //   - writes the samples' rows, crystals in order, to the stage area (row =
 //     sample - t0, pitch srow), for samples of the tile proper; two byte
 //     permutes turn (crystal x, x+1) x (sample t, t+1) into row words.
+// kRows: the slot holds rows by row copies (see row_load).
+template <bool kRows = false>
 __device__ __forceinline__ void sum_pass_step(const KArgs &a, const TileInfo &T, uint32_t slot_s, int it,
                                               int nbt, uint8_t *abyte, int32_t *blocksum, int32_t *sarr,
                                               unsigned char *stage, int lane)
@@ -306,7 +425,9 @@ __device__ __forceinline__ void sum_pass_step(const KArgs &a, const TileInfo &T,
     uint32_t *row0 = reinterpret_cast<uint32_t *>(stage + (st0 || st1 ? (t - T.t0) * a.srow : 0));
     uint32_t *row1 = row0 + (a.srow >> 2);
     int acc0 = 0, acc1 = 0;
-    if (have) {
+    if constexpr (kRows) {
+        sum_rows(a, T, slot_s, it, lane, acc0, acc1);
+    } else if (have) {
         // even and odd crystals in separate accumulators: two dependency chains
         // of X/2 dp2a each instead of one of X
         int acc0b = 0, acc1b = 0;
@@ -589,7 +710,7 @@ __device__ __forceinline__ unsigned read_status(const TileStatus *st, long long 
 // latest entries up to and including the first one that is not fully marked.
 // Bounded: gives up after a.wait_ns or once another CTA has flagged a
 // timeout, returning a poisoned prefix.
-__device__ Agg look_back_in(const KArgs &a, const TileStatus *st, long long tile, int lane, unsigned *stats = nullptr)
+static __device__ Agg look_back_in(const KArgs &a, const TileStatus *st, long long tile, int lane, unsigned *stats = nullptr)
 {
     constexpr int PER = 4, BIG = 1 << 20;
     long long pos = tile - 1;

@@ -184,7 +184,11 @@ __device__ __forceinline__ bool wait_counter_ge(const KArgs &a, const unsigned l
 // tiles compacted, and its aggregate is published with a release store and a
 // valid bit for the scanner.
 // kHaloFree: the count pass loads the tile proper only (see complete_tile).
-template <int TW, bool kFused, int NS = 2, bool kHaloFree = false>
+// kRows: tiles come in row by row (see row_load), each sum warp copying its share
+// of the rows of tile j + NS once all are done with tile j.  Tile records are then
+// kept by j mod 2 NS: when the marks warp has finished tile j it decodes tile j +
+// 2 NS into its place, so that no sum warp waits for a pedestal sum.
+template <int TW, bool kFused, int NS = 2, bool kHaloFree = false, bool kRows = false>
 __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, long long first, long long G)
 {
     constexpr int NWT = TW / 32, NBT = TW / 8;
@@ -208,7 +212,7 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
 
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
-            mbar_init(full + s, 1);
+            mbar_init(full + s, kRows ? 33 * NSW : 1);
             mbar_init(sums + s, NSW);
             mbar_init(mdone + s, 1);
         }
@@ -216,6 +220,10 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
     }
     __syncthreads();
     const long long total = plan.fts[a.n_fills];
+    if constexpr (kRows) {
+        if (tid < 2 * NS && first + tid * G < total) decode_tile<TW>(a, first + tid * G, tinfo[tid], plan.fts, plan.lens);
+        __syncthreads();
+    }
     const int n_steps = (a.ew + 63) / 64;
     constexpr int kSumThreads = 32 * NSW;
 
@@ -240,21 +248,37 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
         }
         trace_stamp(a, tile, 1);
     };
+    auto start_rows = [&](long long j, int s) {  // kRows: every sum warp
+        const TileInfo T = tinfo[j % (2 * NS)];
+        row_load(a, T, slot0 + (size_t)s * a.slot_bytes, a.rs, T.t0 - a.hl, 0, a.ew, warp, NSW, lane);
+        row_load_arrive(full + s);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full + s);  // samples stored one by one come before this
+        if (tid == 0) {
+            trace_stamp(a, T.tile, 0);
+            trace_value(a, T.tile, 10, sm_id());
+            trace_value(a, T.tile, 11, TW);
+            trace_stamp(a, T.tile, 1);
+        }
+    };
     auto slot_wait = [&](uint64_t *bar, uint32_t parity) {
         return kFused ? warp_wait_abortable(a, bar, parity) : warp_wait(bar, parity);
     };
 
     if (warp < NSW) {
-        if (tid == 0)
+        if (kRows || tid == 0)
             for (int k = 0; k < NS; ++k)
-                if (first + k * G < total) start_load(first + k * G, k);
+                if (first + k * G < total) {
+                    if constexpr (kRows) start_rows(k, k);
+                    else start_load(first + k * G, k);
+                }
         for (long long j = 0;; ++j) {
             const long long tile = first + j * G;
             if (tile >= total) break;
             const int s = (int)(j % NS);
             const uint32_t par = (uint32_t)((j / NS) & 1);
             unsigned char *slot = slot0 + (size_t)s * a.slot_bytes;
-            if (a.use_tma) {
+            if (kRows || a.use_tma) {
                 if (!slot_wait(full + s, par)) {
                     if (lane == 0) set_status_bit(a, DAQ_DEV_TIMEOUT);
                     break;
@@ -269,18 +293,27 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
                 if (lane == 0) set_status_bit(a, DAQ_DEV_TIMEOUT);
                 break;
             }
-            const TileInfo T = tinfo[s];
+            const TileInfo T = tinfo[kRows ? (int)(j % (2 * NS)) : s];
             if (tid == 0) {
                 trace_stamp(a, T.tile, 2);
-                tinfo_m[s] = T;
+                if (!kRows) tinfo_m[s] = T;
             }
             const uint32_t slot_s = smem_addr(slot);
             for (int it = warp; it < n_steps; it += NSW)
-                sum_pass_step(a, T, slot_s, it, NBT, abyte0 + 128 * s, blocksum0 + NBT * s,
-                              sarr0 + (a.need_sarr ? TW * s : 0), nullptr, lane);
+                sum_pass_step<kRows>(a, T, slot_s, it, NBT, abyte0 + 128 * s, blocksum0 + NBT * s,
+                                     sarr0 + (a.need_sarr ? TW * s : 0), nullptr, lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(sums + s);
-            if (tid == 0) {
+            if constexpr (kRows) {
+                if (tid == 0) trace_stamp(a, T.tile, 3);
+                if (tile + NS * G < total) {
+                    if (!warp_wait(sums + s, par)) {
+                        if (lane == 0) set_status_bit(a, DAQ_DEV_TIMEOUT);
+                        break;
+                    }
+                    start_rows(j + NS, s);
+                }
+            } else if (tid == 0) {
                 trace_stamp(a, T.tile, 3);
                 // slot s takes tile j + NS once every sum warp is done with tile j
                 if (tile + NS * G < total) {
@@ -293,6 +326,7 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
                 }
             }
         }
+        if (kRows) row_load_wait();  // a warp that stopped early has copies in flight
         // a warp that stopped early leaves loads in flight: they land before
         // the CTA may exit (a slot's latest phase; immediate when consumed)
         if (kFused && tid == 0)
@@ -309,7 +343,12 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
                 if (lane == 0) set_status_bit(a, DAQ_DEV_TIMEOUT);
                 break;
             }
-            const TileInfo T = tinfo_m[s];
+            const TileInfo T = kRows ? tinfo[j % (2 * NS)] : tinfo_m[s];
+            // kRows: the record of tile j has been read; tile j + 2 NS takes its place
+            auto decode_ahead = [&] {
+                if (kRows && lane == 0 && tile + 2 * NS * G < total)
+                    decode_tile<TW>(a, tile + 2 * NS * G, tinfo[j % (2 * NS)], plan.fts, plan.lens);
+            };
             if (kHaloFree) {
                 // internal marks of the tile and its first / last crossing; the
                 // scan adds the marks that crossings of neighbouring tiles reach
@@ -325,6 +364,7 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
                                   (int)(T.t0 / TW), (int)T.len);
                 if (!skip_q) q_partial(a, T, blocksum0 + NBT * s, sarr0 + (a.need_sarr ? TW * s : 0), lane, 32);
                 __syncwarp();
+                decode_ahead();
                 if (lane == 0) mbar_arrive(mdone + s);
                 continue;
             }
@@ -358,6 +398,7 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
             }
             if (!skip_q) q_partial(a, T, blocksum0 + NBT * s, sarr0 + (a.need_sarr ? TW * s : 0), lane, 32);
             __syncwarp();
+            decode_ahead();
             if (lane == 0) mbar_arrive(mdone + s);
         }
     }
@@ -365,13 +406,13 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
 
 // NS = 2: two CTAs per SM; NS = 3: one CTA per SM with 16 sum warps, for
 // extended tiles too wide for two CTAs' slots to fit.  HF: halo-free.
-template <int TW, int NS, bool HF>
+template <int TW, int NS, bool HF, bool ROWS>
 __global__ void __launch_bounds__(count_threads<NS>(), NS == 2 ? 2 : 1) daq_count_kernel(const __grid_constant__ KArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     pdl_wait();     // the prepare kernel's plan, pedestals and resets
     pdl_trigger();  // the scan may be scheduled as CTAs finish
-    count_role<TW, false, NS, HF>(a, smem, blockIdx.x, gridDim.x);
+    count_role<TW, false, NS, HF, ROWS>(a, smem, blockIdx.x, gridDim.x);
 }
 
 // ============================================================================ scan of the aggregates
@@ -555,8 +596,11 @@ __global__ void __launch_bounds__(kScanThreads) daq_scan_kernel(const __grid_con
 // owns columns c = 64 it + 2L, c + 1 of the tile proper; a marked sample's row
 // goes to byte phase + r * 2X of the stage, r = its rank among the tile's
 // marked samples.
+// kRows: the slot holds rows by row copies, row 0 at byte phase ph0.
+template <bool kRows>
 __device__ __forceinline__ void compact_step(const KArgs &a, uint32_t slot_s, int it, int nt, const uint32_t *wm,
-                                             const int32_t *wmb, unsigned char *stage, int phase, int lane)
+                                             const int32_t *wmb, unsigned char *stage, int phase, int lane,
+                                             uint32_t ph0)
 {
     const int X = a.n_xtal;
     const int c = 64 * it + 2 * lane;
@@ -570,7 +614,30 @@ __device__ __forceinline__ void compact_step(const KArgs &a, uint32_t slot_s, in
     const int k = (c >= a.boxw_b) + (c >= 2 * a.boxw_b) + (c >= 3 * a.boxw_b) + (c >= 4 * a.boxw_b);
     const uint32_t base = slot_s + (uint32_t)(k * a.box_stride_b + 2 * (c - k * a.boxw_b));
     unsigned char *row0 = stage + phase + (size_t)r0 * 2 * X, *row1 = stage + phase + (size_t)r1 * 2 * X;
-    if (!(X & 1)) {
+    if constexpr (kRows) {
+        // a row whose phase is odd in samples: the two samples lie in two words
+        const uint32_t dph = 2u * (uint32_t)a.n_samples, at = slot_s + 2 * c;
+        const bool odd0 = ph0 & 2u, odd1 = (ph0 + dph) & 2u;  // rows of even and of odd index
+        auto pair = [&](int x, bool odd) {
+            const uint32_t p = at + (uint32_t)(x * a.rs_b) + ((ph0 + x * dph) & 12u);
+            const uint32_t w = lds_u32(p);
+            return odd ? __funnelshift_r(w, lds_u32(p + 4), 16) : w;
+        };
+        if (!(X & 1)) {
+#pragma unroll 3
+            for (int x = 0; x < X; x += 2) {
+                const uint32_t w0 = pair(x, odd0), w1 = pair(x + 1, odd1);
+                if (m0) *reinterpret_cast<uint32_t *>(row0 + 2 * x) = __byte_perm(w0, w1, 0x5410);
+                if (m1) *reinterpret_cast<uint32_t *>(row1 + 2 * x) = __byte_perm(w0, w1, 0x7632);
+            }
+        } else {
+            for (int x = 0; x < X; ++x) {
+                const uint32_t w0 = pair(x, x & 1 ? odd1 : odd0);
+                if (m0) *reinterpret_cast<uint16_t *>(row0 + 2 * x) = (uint16_t)(w0 & 0xffffu);
+                if (m1) *reinterpret_cast<uint16_t *>(row1 + 2 * x) = (uint16_t)(w0 >> 16);
+            }
+        }
+    } else if (!(X & 1)) {
 #pragma unroll 3
         for (int x = 0; x < X; x += 2) {
             const uint32_t w0 = lds_u32(base + (uint32_t)(x * a.rs_b));
@@ -634,7 +701,11 @@ __device__ __forceinline__ void plain_tile_load_b(const KArgs &a, const TileInfo
 // kFused: a tile's marks, record and prefix are read once the scanner has
 // passed it (L1-bypassing loads: other CTAs wrote them during this launch), and
 // each tile staged is counted in the compacted counter.
-template <int TW, bool kFused, bool kSparse = false>
+// kRows: a tile comes in row by row (see row_load), from its first marked
+// 64-sample step to its last, every warp copying its share of the rows (the box
+// mask handed between the warps is then the mask of marked steps, and warp 0
+// decodes the next tile ahead, into the other of two records).
+template <int TW, bool kFused, bool kSparse = false, bool kRows = false>
 __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem, long long first, long long G)
 {
     constexpr int NWT = TW / 32;
@@ -656,6 +727,7 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
     uint32_t *s_boxes = reinterpret_cast<uint32_t *>(lens_s + kPlanSmem);  // boxes of the CTA's next tile
     // kSparse: the CTA's next tile, when tile + G holds no marked sample
     long long *s_next = reinterpret_cast<long long *>((reinterpret_cast<uintptr_t>(s_boxes + 1) + 7) & ~uintptr_t(7));
+    TileInfo *tinfo_r = reinterpret_cast<TileInfo *>(s_next + 1);  // kRows: [2]
     const PlanView plan = cache_plan(a, fts_s, lens_s, tid, nthr);
     if (tid == 0) {
         mbar_init(bar, 1);
@@ -666,7 +738,7 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
     const TileRec *recs = reinterpret_cast<const TileRec *>(a.recs);
     const TileExcl *exs = reinterpret_cast<const TileExcl *>(a.excl);
     const uint32_t one_box = (uint32_t)X * (uint32_t)a.rs_b;
-    const uint32_t all_boxes = (1u << a.nbox_b) - 1u;
+    const uint32_t all_boxes = (1u << (kRows ? (TW + 63) / 64 : a.nbox_b)) - 1u;
     // Boxes of a tile to load: those covering a 64-sample step its count record
     // marks (box k holds columns [k boxw, (k + 1) boxw)); the single-launch
     // form's records may not be published yet: all.
@@ -676,6 +748,7 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
     auto boxes_of = [&](uint32_t flags) -> uint32_t {
         if (flags == ~0u) return all_boxes;
         const uint32_t steps = flags >> kRecStepShift;
+        if constexpr (kRows) return steps;
         uint32_t boxes = 0;
         for (int k = 0; k < a.nbox_b; ++k) {
             const int s0 = (k * a.boxw_b) >> 6, s1 = ((k + 1) * a.boxw_b - 1) >> 6;
@@ -723,6 +796,14 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
         }
     };
 
+    int cur = 0;  // kRows: the tile's record of tinfo_r
+    auto start_rows = [&](uint32_t steps) {  // kRows: every warp
+        if (steps == 0) return;
+        const TileInfo T = tinfo_r[cur];
+        const int c0 = 64 * (__ffs(steps) - 1), c1 = min(64 * (32 - __clz(steps)), TW);
+        row_load(a, T, slot, a.rs_b, T.t0, c0, c1, warp, nwarps, lane);
+    };
+
     // warp 0's inputs of the next tile, in registers, and (lane 0) the record
     // flags of the tile after it (kSparse: and its marked samples); false if
     // the wait gave up
@@ -766,7 +847,11 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
     TileExcl ne{0, 0, 0};
     int in_ok = 1;
     if (first < total) {
-        if (tid == 32) {
+        if constexpr (kRows) {
+            if (tid == 0) decode_tile<TW>(a, first, tinfo_r[0], plan.fts, plan.lens, false);
+            __syncthreads();
+            start_rows(boxes_of(flags_of(first)));
+        } else if (tid == 32) {
             start_load(first, boxes_of(flags_of(first)));
             load_pending = kFused;
         }
@@ -775,21 +860,24 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
     for (long long tile = first; tile < total;) {
         int moved = 0;  // kSparse, warp 0: the next tile is not tile + G (it is in s_next)
         if (__syncthreads_or(!in_ok)) break;  // tinfo holds this tile; warp 0 has its inputs
-        const TileInfo T = *tinfo;
-        if (!a.use_tma) plain_tile_load_b(a, T, slot, tid, nthr);
+        const TileInfo T = kRows ? tinfo_r[cur] : *tinfo;
+        if (!kRows && !a.use_tma) plain_tile_load_b(a, T, slot, tid, nthr);
         if (warp == 0) {
             const Agg g = words_from_marks<TW>(nMt, (nr.flags >> 1) & 1, (nr.flags >> 2) & 1,
                                                (int)(T.t_end - T.t0), W, nullptr, lane);
             uint32_t fl = nfl2;
+            long long next = tile + G;  // kRows: the tile decoded ahead
             if constexpr (kSparse) {
                 if (tile + G < total && __shfl_sync(kFull, nm2, 0) == 0) {
                     // tile + G holds no marked sample: find the CTA's next one
                     long long nt;
                     find_next(tile + 2 * G, nt, fl);
                     moved = 1;
+                    next = nt;
                     if (lane == 0) *s_next = nt;
                 }
             }
+            if (kRows && lane == 0 && next < total) decode_tile<TW>(a, next, tinfo_r[cur ^ 1], plan.fts, plan.lens, false);
             if (lane == 0) {
                 *s_boxes = boxes_of(fl);  // read with this tile's inputs; the next load uses it
                 Agg ex;
@@ -806,7 +894,10 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
                 }
             }
         }
-        if (a.use_tma) {
+        if constexpr (kRows) {
+            row_load_wait();
+            __syncthreads();
+        } else if (a.use_tma) {
             const bool ok = mbar_wait_bounded(bar, phase_bit, kWaitLimitNs);
             if (ok) load_pending = false;
             phase_bit ^= 1u;
@@ -823,8 +914,9 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
         const long long gs = ex.m * rb;
         const int phase = (int)(gs & 15);
         const int nt = (int)(T.t_end - T.t0);
+        const uint32_t ph0 = kRows ? row_phase0(a, (long long)T.f * a.n_calo + T.c, T.t0) : 0u;
         for (int it = warp; it < (nt + 63) / 64; it += nwarps)
-            compact_step(a, smem_addr(slot), it, nt, W.m, W.mb, stage, phase, lane);
+            compact_step<kRows>(a, smem_addr(slot), it, nt, W.m, W.mb, stage, phase, lane, ph0);
         // rows staged; the slot is free
         long long next = tile + G;
         if constexpr (kSparse) {
@@ -834,7 +926,10 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
         }
         if (kFused && tid == 0) atomicAdd(compacted_ctr(a), 1ull);
         if (next < total) {
-            if (tid == 32) {
+            if constexpr (kRows) {
+                cur ^= 1;
+                start_rows(*s_boxes);
+            } else if (tid == 32) {
                 start_load(next, *s_boxes);
                 load_pending = kFused && a.use_tma;  // the single-launch form may stop before waiting for it
             }
@@ -885,13 +980,13 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
     if (tid == 32 && load_pending) mbar_wait_bounded(bar, phase_bit, kWaitLimitNs);  // left early: let it land
 }
 
-template <int TW, bool kSparse>
+template <int TW, bool kSparse, bool ROWS>
 __global__ void __launch_bounds__(256, 2) daq_compact_kernel(const __grid_constant__ KArgs a)
 {
     pdl_wait();                // every tile's prefix
     if (aborted(a)) return;    // the scan gave up: its prefixes are incomplete
     extern __shared__ __align__(128) unsigned char smem[];
-    compact_role<TW, false, kSparse>(a, smem, blockIdx.x, gridDim.x);
+    compact_role<TW, false, kSparse, ROWS>(a, smem, blockIdx.x, gridDim.x);
 }
 
 // ============================================================================ single-launch form
