@@ -12,24 +12,8 @@
 // row differences of a crystal are small (noise, pulse edges) and a block's
 // crystal column typically needs a few bits per sample instead of 16.
 //
-// One warp per block at a time, blocks b, b + W, ... (W warps in the grid).
-// Each warp keeps two block buffers in shared memory: while it works on one,
-// a bulk copy (one instruction, completing on the buffer's mbarrier) brings
-// in its next block, so the global load latency overlaps the work.  The size
-// pass puts lanes on crystal columns: a lane walks its
-// column down the 32 rows OR-ing the zigzag differences (the bit length of the
-// OR is that of the maximum: the column's width) and the block's size
-// follows.  An exclusive scan of the block sizes (three kernels) gives the
-// offsets.  The write pass puts lanes on rows (row pitch an odd number of
-// words, so a warp reading one crystal down 32 rows hits 32 banks): one
-// shuffle forms a column's differences and one 32 x 32 bit transpose across
-// the warp turns them into bit planes held by lanes in stream order, shared
-// by two or four columns when their widths allow.  The decoder puts lanes on
-// crystal columns (see unpack_kernel).  (One ballot per plane, the
-// first form, took 2.7x as long: the integer pipe ran out.  A single pass
-// whose warps found their block's place by decoupled look-back was slower
-// still: with thousands of one-block warps in flight the nearest published
-// prefix lies hundreds of blocks back.)
+// The encoder is one pass over the pool (pack_kernel), the decoder one over the
+// stream (unpack_kernel); in both a lane owns two crystal columns of a block.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -41,38 +25,13 @@
 namespace daq_pack {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kWarps = 8;
-constexpr int kThreads = 32 * kWarps;
 constexpr int kMaxX = 64;
 constexpr uint32_t kMagic = 0x50514144u;
-constexpr int kScanPer = 4;
-constexpr int kScanChunk = kThreads * kScanPer;
-constexpr uint64_t kWaitNs = 4000000000ull;  // a block copy not landed after this: give up (error word)
+constexpr uint64_t kWaitNs = 4000000000ull;  // a block copy not landed, or an earlier chunk not heard of, after this: give up
 
 __device__ __forceinline__ uint32_t zigzag(int32_t d) { return ((uint32_t)d << 1) ^ (uint32_t)(d >> 31); }
 
 __device__ __forceinline__ int32_t unzigzag(uint32_t z) { return (z & 1u) ? -(int32_t)((z + 1u) >> 1) : (int32_t)(z >> 1); }
-
-// Per 16-bit half, modulo 2^16: v - p (no borrow crosses the halves).
-__device__ __forceinline__ uint32_t sub16x2(uint32_t v, uint32_t p)
-{
-    return ((v | 0x80008000u) - (p & 0x7fff7fffu)) ^ ((v ^ ~p) & 0x80008000u);
-}
-
-// Per 16-bit half: zigzag(d) = 2d for d >= 0, -2d - 1 else, i.e. (d << 1) ^
-// (the half's sign spread over it); the sign comes from a byte permute that
-// replicates the top bit of bytes 1 and 3.
-__device__ __forceinline__ uint32_t zigzag16x2(uint32_t d)
-{
-    uint32_t sgn;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(sgn) : "r"(d), "r"(0u), "r"(0xbb99u));
-    return ((d << 1) & 0xfffefffeu) ^ sgn;
-}
-
-// A warp's shared rows: the block's 32 rows back to back (row pitch X), as in
-// the pool.  Reading one crystal down the rows strides X int16 per lane, which
-// is conflict-free whenever X/2 is odd (54 crystals: 27 words per row).
-constexpr int kBlockElems = 32 * kMaxX;
 
 // Copy block b's rows (16-byte vectors; the pool and every block start are
 // 16-byte aligned) into the warp's shared rows, rows past the pool's end
@@ -93,440 +52,12 @@ __device__ __forceinline__ int load_block(const int16_t *pool, long long rows, i
     return nv;
 }
 
-// Per-warp pipeline of 32-row blocks in dynamic shared memory: two buffers
-// of 64 X bytes (a block's rows back to back, row pitch X, as in the pool:
-// reading one crystal down the rows strides X int16 per lane, conflict-free
-// whenever X/2 is odd, as for 54 crystals), then `extra` bytes of the
-// caller's, then two mbarriers.  Blocks below nfull (32 real rows) come in by
-// bulk copy, one block ahead; the last block, when it is shorter, is copied by
-// the lanes with its padding rows.  `wait` returns false when a copy did not
-// land within kWaitNs; `drain` waits (bounded) for copies still in flight, so
-// that the warp may leave.
-struct BlockPipe {
-    unsigned char *base, *extra;
-    uint64_t *bar;
-    int bufb;               // bytes of one buffer (64 X)
-    uint32_t pend = 0;      // lane 0: buffers with a copy issued and not waited for
-    uint32_t par = 0;       // lane 0: bit s = phase parity of buffer s's pending copy
-    uint32_t next_par = 0;  // bit s = phase parity the next wait on buffer s expects
-
-    static __host__ __device__ size_t bytes(int X, int extra) { return 2 * 64 * (size_t)X + (size_t)extra + 16; }
-
-    __device__ BlockPipe(unsigned char *b, int X, int extra_bytes, int lane)
-        : base(b), extra(b + 128 * X), bar(reinterpret_cast<uint64_t *>(b + 128 * X + extra_bytes)), bufb(64 * X)
-    {
-        if (lane == 0) {
-            daq::mbar_init(bar, 1);
-            daq::mbar_init(bar + 1, 1);
-            daq::fence_mbar_init();
-        }
-        __syncwarp();
-    }
-    __device__ int16_t *buf(int s) const { return reinterpret_cast<int16_t *>(base + s * bufb); }
-    // lane 0: start the copy of full block b into buffer s (the warp is done with it)
-    __device__ void issue(const int16_t *pool, int X, long long b, int s)
-    {
-        daq::fence_proxy_async_smem();
-        daq::mbar_arrive_expect_tx(bar + s, (uint32_t)bufb);
-        daq::bulk_g2s(buf(s), pool + 32ll * b * X, (uint32_t)bufb, bar + s);
-        pend |= 1u << s;
-        par = (par & ~(1u << s)) | (next_par & (1u << s));
-    }
-    // every lane: block b's rows are in buffer s
-    __device__ bool wait(const int16_t *pool, long long rows, int X, long long b, long long nfull, int s, int lane)
-    {
-        if (b < nfull) {
-            if (!daq::mbar_wait_bounded(bar + s, (next_par >> s) & 1u, kWaitNs)) return false;
-            next_par ^= 1u << s;
-            pend &= ~(1u << s);
-        } else {
-            load_block(pool, rows, X, b, buf(s), lane);
-        }
-        return true;
-    }
-    // lane 0: wait (bounded) for copies still in flight, so that the warp may leave
-    __device__ void drain()
-    {
-        for (int s = 0; s < 2; ++s)
-            if (pend & (1u << s)) daq::mbar_wait_bounded(bar + s, (par >> s) & 1u, kWaitNs);
-    }
-};
-
-// Block sizes, and the width of every crystal column (widths[b][x]).  Lanes
-// take crystal columns here: lane x walks its column down the block's 32 rows
-// (consecutive lanes read consecutive samples of a row: no bank conflict),
-// OR-ing the zigzag differences in a register, so a column costs a few
-// instructions per row shared by 32 columns instead of a shuffle and a
-// reduction of its own.
-__global__ void __launch_bounds__(kThreads) pack_size_kernel(const int16_t *pool, long long rows, int X,
-                                                             long long nb, unsigned long long *sizes,
-                                                             uint8_t *widths, int *perr)
-{
-    extern __shared__ __align__(16) unsigned char dsm[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    BlockPipe pipe(dsm + warp * BlockPipe::bytes(X, 0), X, 0, lane);
-    const long long nfull = rows / 32, W = (long long)gridDim.x * kWarps;
-    long long b = (long long)blockIdx.x * kWarps + warp;
-    if (lane == 0 && b < nfull) pipe.issue(pool, X, b, 0);
-    for (int it = 0; b < nb; b += W, ++it) {
-        const int s = it & 1;
-        if (lane == 0 && b + W < nfull) pipe.issue(pool, X, b + W, s ^ 1);
-        if (!pipe.wait(pool, rows, X, b, nfull, s, lane)) {
-            if (lane == 0) atomicOr(perr, 1);
-            break;
-        }
-        const int16_t *sm = pipe.buf(s);
-        unsigned words = 0;
-        for (int x = lane; x < X; x += 32) {
-            const int16_t *col = sm + x;
-            int32_t prev = col[0];
-            uint32_t acc = 0;
-#pragma unroll
-            for (int r = 1; r < 32; ++r) {
-                const int32_t v = col[r * X];
-                acc |= zigzag(v - prev);
-                prev = v;
-            }
-            const int w = 32 - __clz(acc);  // 0 for acc = 0
-            widths[b * X + x] = (uint8_t)w;
-            words += 1u + (unsigned)w;
-        }
-        words = __reduce_add_sync(kFull, words);
-        if (lane == 0) sizes[b] = 4ull * words;
-        __syncwarp();
-    }
-    if (lane == 0) pipe.drain();
-}
-
-// ------------------------------------------------------------------ exclusive scan of the block sizes
-__global__ void __launch_bounds__(kThreads) scan_reduce_kernel(const unsigned long long *v, long long n,
-                                                               unsigned long long *chunk)
-{
-    __shared__ unsigned long long s[kWarps];
-    const long long base = (long long)blockIdx.x * kScanChunk + threadIdx.x * kScanPer;
-    unsigned long long t = 0;
-    for (int i = 0; i < kScanPer; ++i)
-        if (base + i < n) t += v[base + i];
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(kFull, t, d);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long a = 0;
-        for (int w = 0; w < kWarps; ++w) a += s[w];
-        chunk[blockIdx.x] = a;
-    }
-}
-
-// One block: chunk sums -> exclusive prefixes (in place); chunk[n_chunks] = total.
-__global__ void __launch_bounds__(1024) scan_top_kernel(unsigned long long *chunk, long long n_chunks)
-{
-    __shared__ unsigned long long s[32];
-    __shared__ unsigned long long carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (long long base = 0; base < n_chunks; base += 1024) {
-        const long long i = base + threadIdx.x;
-        const unsigned long long v = i < n_chunks ? chunk[i] : 0ull;
-        unsigned long long x = v;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned long long y = __shfl_up_sync(kFull, x, d);
-            if (lane >= d) x += y;
-        }
-        if (lane == 31) s[warp] = x;
-        __syncthreads();
-        unsigned long long pre = carry;
-        for (int w = 0; w < warp; ++w) pre += s[w];
-        if (i < n_chunks) chunk[i] = pre + x - v;
-        __syncthreads();
-        if (threadIdx.x == 1023) carry = pre + x;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) chunk[n_chunks] = carry;
-}
-
-// offsets[b] = exclusive prefix (workspace, and the stream's table when it
-// fits), offsets[nb] = payload size, *out_bytes = whole stream size.
-__global__ void __launch_bounds__(kThreads) scan_apply_kernel(const unsigned long long *v, long long n,
-                                                              const unsigned long long *chunk,
-                                                              unsigned long long *offs, unsigned char *out,
-                                                              long long cap, long long *out_bytes, const int *perr)
-{
-    __shared__ unsigned long long s[kWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long base = (long long)blockIdx.x * kScanChunk + threadIdx.x * kScanPer;
-    unsigned long long loc[kScanPer], t = 0;
-    for (int i = 0; i < kScanPer; ++i) {
-        loc[i] = base + i < n ? v[base + i] : 0ull;
-        t += loc[i];
-    }
-    unsigned long long x = t;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned long long y = __shfl_up_sync(kFull, x, d);
-        if (lane >= d) x += y;
-    }
-    if (lane == 31) s[warp] = x;
-    __syncthreads();
-    unsigned long long pre = chunk[blockIdx.x];
-    for (int w = 0; w < warp; ++w) pre += s[w];
-    pre += x - t;
-    const long long table = 16;  // the offsets table starts after the 16-byte header
-    for (int i = 0; i < kScanPer; ++i) {
-        const long long k = base + i;  // entries 0..n (entry n: the payload size)
-        if (k <= n) {
-            offs[k] = pre;
-            if (table + 8 * k + 8 <= cap) reinterpret_cast<unsigned long long *>(out + table)[k] = pre;
-            if (k == n) *out_bytes = *perr ? -1 : 16 + 8 * (n + 1) + (long long)pre;  // -1: the size pass gave up
-        }
-        pre += loc[i];
-    }
-}
-
-// 32 x 32 bit transpose across the warp: lane j receives bit j of every lane's
-// x (bit i of the result = bit j of lane i's x).  Five stages of the recursive
-// block swap: at stage s the lane pairs (l, l ^ s) exchange the off-diagonal
-// s x s blocks - the lane with bit s clear keeps the bits whose index has bit
-// s clear (mask m) and takes its partner's such bits shifted up by s, the
-// other keeps ~m and takes its partner's ~m bits shifted down by s.  Each
-// shift is a rotation (funnel shift) whose unwanted bits the select drops, so
-// a stage is one shuffle, one rotation and one bitwise select.
-struct Transpose {
-    uint32_t keep[5];
-    int rot[5];
-    __device__ __forceinline__ explicit Transpose(int lane)
-    {
-        constexpr uint32_t kMask[5] = {0x0000ffffu, 0x00ff00ffu, 0x0f0f0f0fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-        for (int t = 0; t < 5; ++t) {
-            const int sft = 16 >> t;
-            const bool low = (lane & sft) == 0;
-            keep[t] = low ? kMask[t] : ~kMask[t];
-            rot[t] = low ? sft : 32 - sft;
-        }
-    }
-    __device__ __forceinline__ uint32_t operator()(uint32_t x) const
-    {
-#pragma unroll
-        for (int t = 0; t < 5; ++t) {
-            const uint32_t y = __shfl_xor_sync(kFull, x, 16 >> t);
-            const uint32_t r = __funnelshift_l(y, y, rot[t]);
-            x = (x & keep[t]) | (r & ~keep[t]);
-        }
-        return x;
-    }
-    // two independent transposes, stage by stage (their shuffles overlap)
-    __device__ __forceinline__ void two(uint32_t &x, uint32_t &z) const
-    {
-#pragma unroll
-        for (int t = 0; t < 5; ++t) {
-            const uint32_t y = __shfl_xor_sync(kFull, x, 16 >> t);
-            const uint32_t w = __shfl_xor_sync(kFull, z, 16 >> t);
-            x = (x & keep[t]) | (__funnelshift_l(y, y, rot[t]) & ~keep[t]);
-            z = (z & keep[t]) | (__funnelshift_l(w, w, rot[t]) & ~keep[t]);
-        }
-    }
-};
-
-// Crystal columns go through the transpose four at a time when all four
-// widths are <= 7 (the common case for noise-dominated island rows), else in
-// pairs when both are <= 15, else alone.  A group of G = 8, 16 or 32 lanes
-// serves one column: its z << 1 sits at bit G g of the transposed word, so
-// lane G g + k + 1 receives plane k and the group's first lane, which receives
-// zeros, carries the head word instead.  One store then writes every column's
-// words, which lie back to back: the head, then the planes.
-// - Four: byte g of (w4 + 0x01010101) * 0x01010100 is the words of the columns
-//   before g (w4 = the four widths as bytes); lane 0 broadcasts the first
-//   samples two to a word.
-// - Alone (a width of 16 or 17: a difference of at least 2^14).
-// kPairs (even X): in the four-column path a lane reads its row's crystals two
-// to a 32-bit word and forms both differences and zigzag codes at once, in
-// 16-bit halves (exact there: every difference is within +-64).
-// A block copy that does not land within kWaitNs sets *out_bytes to -1.
-template <bool kPairs>
-__global__ void __launch_bounds__(kThreads, 4) pack_write_kernel(const int16_t *pool, long long rows, int X, long long nb,
-                                                              const unsigned long long *offs, const uint8_t *widths,
-                                                              unsigned char *out, long long cap, long long *out_bytes)
-{
-    extern __shared__ __align__(16) unsigned char dsm[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    BlockPipe pipe(dsm + warp * BlockPipe::bytes(X, kMaxX), X, kMaxX, lane);
-    uint8_t *wsm = pipe.extra;  // widths of the block being written
-    const Transpose transpose(lane);
-    const int k16 = lane & 15, k8 = lane & 7;
-    const bool hi16 = lane >= 16;
-    const int g4 = lane >> 3, g8 = 8 * g4;  // four-column group of this lane, its byte
-    uint32_t *out32 = reinterpret_cast<uint32_t *>(out);
-    const long long head = 16 + 8 * (nb + 1);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && cap >= 16) {
-        out32[0] = kMagic;
-        out32[1] = (uint32_t)X;
-        reinterpret_cast<unsigned long long *>(out)[1] = (unsigned long long)rows;
-    }
-    const long long nfull = rows / 32, Wn = (long long)gridDim.x * kWarps;
-    long long b = (long long)blockIdx.x * kWarps + warp;
-    int w_lo = 0, w_hi = 0;  // widths of columns lane and lane + 32 of the block to come
-    auto widths_of = [&](long long bb) {
-        w_lo = lane < X ? widths[bb * X + lane] : 0;
-        w_hi = lane + 32 < X ? widths[bb * X + lane + 32] : 0;
-    };
-    if (b < nb) {
-        if (lane == 0 && b < nfull) pipe.issue(pool, X, b, 0);
-        widths_of(b);
-    }
-    for (int it = 0; b < nb; b += Wn, ++it) {
-        const int s = it & 1;
-        if (lane < X) wsm[lane] = (uint8_t)w_lo;
-        if (lane + 32 < X) wsm[lane + 32] = (uint8_t)w_hi;
-        if (b + Wn < nb) {
-            if (lane == 0 && b + Wn < nfull) pipe.issue(pool, X, b + Wn, s ^ 1);
-            widths_of(b + Wn);
-        }
-        if (!pipe.wait(pool, rows, X, b, nfull, s, lane)) {
-            if (lane == 0) *out_bytes = -1;
-            break;
-        }
-        __syncwarp();
-        const int16_t *row = pipe.buf(s) + lane * X;
-        const long long start = head + (long long)offs[b];  // bytes, a multiple of 4
-        uint32_t *dst = out32 + (start >> 2);
-        // words that may be written from the block's start (a block is < 2^11 words)
-        const int room = (int)(max(0ll, min(cap - start, 1ll << 20)) >> 2);
-        int o = 0;  // words of the block written so far
-        auto single = [&](int x) {
-            const int32_t v = row[x];
-            const uint32_t z = zigzag(v - __shfl_up_sync(kFull, v, 1));
-            const int w = wsm[x];
-            const uint32_t planes = transpose(z << 1);
-            const uint32_t word = lane ? planes : ((uint32_t)(uint16_t)v | ((uint32_t)w << 16));
-            if (lane <= w && o + lane < room) dst[o + lane] = word;
-            o += 1 + w;
-        };
-        auto pair = [&](int x) {
-            const int wa = wsm[x], wb = wsm[x + 1];
-            if (max(wa, wb) > 15) {
-                single(x);
-                single(x + 1);
-                return;
-            }
-            const int32_t va = row[x], vb = row[x + 1];
-            const uint32_t za = zigzag(va - __shfl_up_sync(kFull, va, 1));
-            const uint32_t zb = zigzag(vb - __shfl_up_sync(kFull, vb, 1));
-            const uint32_t planes = transpose((za << 1) | (zb << 17));
-            const uint32_t firsts = __shfl_sync(kFull, (uint32_t)(uint16_t)va | ((uint32_t)vb << 16), 0);
-            const int w = hi16 ? wb : wa;
-            const uint32_t hw = (hi16 ? firsts >> 16 : firsts & 0xffffu) | ((uint32_t)w << 16);
-            const int i = o + (hi16 ? 1 + wa : 0) + k16;
-            if (k16 <= w && i < room) dst[i] = k16 ? planes : hw;
-            o += 2 + wa + wb;
-        };
-        // four columns of width <= 7: their z << 1 as bytes, lane 0's samples two to a word
-        auto quad_z = [&](int x, uint32_t &zq, uint32_t &f01, uint32_t &f23) {
-            if constexpr (kPairs) {
-                const uint32_t *row32 = reinterpret_cast<const uint32_t *>(row);
-                const uint32_t v01 = row32[x >> 1], v23 = row32[(x >> 1) + 1];
-                const uint32_t z01 = zigzag16x2(sub16x2(v01, __shfl_up_sync(kFull, v01, 1)));
-                const uint32_t z23 = zigzag16x2(sub16x2(v23, __shfl_up_sync(kFull, v23, 1)));
-                zq = __byte_perm(z01, z23, 0x6420) << 1;  // z < 128: no bit crosses into the next byte
-                f01 = __shfl_sync(kFull, v01, 0);
-                f23 = __shfl_sync(kFull, v23, 0);
-            } else {
-                const int32_t v0 = row[x], v1 = row[x + 1], v2 = row[x + 2], v3 = row[x + 3];
-                const uint32_t z0 = zigzag(v0 - __shfl_up_sync(kFull, v0, 1));
-                const uint32_t z1 = zigzag(v1 - __shfl_up_sync(kFull, v1, 1));
-                const uint32_t z2 = zigzag(v2 - __shfl_up_sync(kFull, v2, 1));
-                const uint32_t z3 = zigzag(v3 - __shfl_up_sync(kFull, v3, 1));
-                zq = (z0 << 1) | (z1 << 9) | (z2 << 17) | (z3 << 25);
-                f01 = __shfl_sync(kFull, (uint32_t)(uint16_t)v0 | ((uint32_t)v1 << 16), 0);
-                f23 = __shfl_sync(kFull, (uint32_t)(uint16_t)v2 | ((uint32_t)v3 << 16), 0);
-            }
-        };
-        // store the words of four columns (widths w4 as bytes) from their transposed planes
-        auto quad_store = [&](uint32_t planes, uint32_t w4, uint32_t f01, uint32_t f23) {
-            const uint32_t fp = g4 < 2 ? f01 : f23;
-            const uint32_t w = (w4 >> g8) & 0xffu;
-            const uint32_t hw = ((g4 & 1) ? fp >> 16 : fp & 0xffffu) | (w << 16);
-            const uint32_t before = (w4 + 0x01010101u) * 0x01010100u;  // byte g: words of columns < g
-            const int i = o + (int)((before >> g8) & 0xffu) + k8;
-            if (k8 <= (int)w && i < room) dst[i] = k8 ? planes : hw;
-            o += (int)(before >> 24) + 1 + (int)(w4 >> 24);
-        };
-        auto narrow = [](uint32_t w4) { return ((w4 + 0x78787878u) & 0x80808080u) == 0u; };  // every width <= 7
-        auto group = [&](int x, uint32_t w4) {
-            if (!narrow(w4)) {
-                pair(x);
-                pair(x + 2);
-                return;
-            }
-            uint32_t zq, f01, f23;
-            quad_z(x, zq, f01, f23);
-            quad_store(transpose(zq), w4, f01, f23);
-        };
-        int x = 0;
-        for (; x + 7 < X; x += 8) {  // two groups of four: both narrow, their transposes overlap
-            const uint32_t w4a = *reinterpret_cast<const uint32_t *>(wsm + x);
-            const uint32_t w4b = *reinterpret_cast<const uint32_t *>(wsm + x + 4);
-            if (narrow(w4a) && narrow(w4b)) {
-                uint32_t za, fa01, fa23, zb, fb01, fb23;
-                quad_z(x, za, fa01, fa23);
-                quad_z(x + 4, zb, fb01, fb23);
-                transpose.two(za, zb);
-                quad_store(za, w4a, fa01, fa23);
-                quad_store(zb, w4b, fb01, fb23);
-            } else {
-                group(x, w4a);
-                group(x + 4, w4b);
-            }
-        }
-        for (; x + 3 < X; x += 4) group(x, *reinterpret_cast<const uint32_t *>(wsm + x));
-        for (; x + 1 < X; x += 2) pair(x);
-        if (x < X) single(x);
-        __syncwarp();
-    }
-    if (lane == 0) pipe.drain();
-}
-
-// ------------------------------------------------------------------ decoder
-// Bound by instruction issue and, at the end, by HBM (61% of its rate).  Lanes
-// own crystal columns, two neighbouring ones each (np = ceil(X / 2) lanes a
-// block, nsub = 32 / np blocks side by side), so a column's bit planes become
-// samples inside one lane: seven three-input operations undo the zigzag on the
-// planes, three stages of bit swaps among eight words (48 operations) turn
-// them into 32 signed bytes (word k, byte j = row 8j + k), and one dp4a a row
-// takes its byte and adds it to the running sample.  A row is one 32-bit store
-// of the lane's two samples; whole blocks leave by bulk copy.  With lanes on
-// rows a column took a 32 x 32 transpose and a prefix sum across the warp, 49
-// instructions a column and warp against 12 here: 12.06 M rows x 54 decoded in
-// 1.19 ms, now 0.34 (the call 1275 -> 383 us).
-// Where the columns' words begin is known only by walking their head words, a
-// chain of X shared-memory loads, so a warp stages the payload of up to G = 4
-// consecutive blocks (16-byte asynchronous copies) and G lanes walk them at
-// once; more would cost occupancy (10 KB a warp, 20 warps an SM).  The next
-// group's payload is brought into L2 while this one is decoded (390 -> 383
-// us).  Undoing the zigzag on bytes after the swaps, copying rows out with
-// 16-byte stores and checking every head word in the walk took 502 us.
-// Columns wider than 8 bits (pulses: 2% of the blocks of a dense fill hold
-// one) take the same swaps on planes 8..15 and add plane 16 bit by bit.
-constexpr int kDecWarps = 4;
-constexpr int kDecThreads = 32 * kDecWarps;
-
-// Lanes, blocks and shared memory of one warp, by the crystal count.
-struct DecPlan {
-    int np, nsub, G, cap;  // cap: bytes of staged payload
-    __host__ __device__ explicit DecPlan(int X)
-    {
-        np = (X + 1) / 2;
-        nsub = 32 / np < 16 ? 32 / np : 16;
-        G = nsub >= 4 ? nsub : nsub == 3 ? 6 : 4;
-        // planes of 6.5 bits a column; one block of the widest columns always fits
-        const int want = G * X * 30, least = X * 72;
-        cap = ((want > least ? want : least) + 15) & ~15;
-    }
-    __host__ __device__ size_t pos_at() const { return (size_t)cap + 32; }  // staged words begin at any 4-byte phase
-    __host__ __device__ size_t out_at(int X) const { return (pos_at() + 2 * (size_t)G * X + 15) & ~size_t(15); }
-    __host__ __device__ size_t bytes(int X) const { return out_at(X) + (size_t)nsub * 64 * X; }
+// ------------------------------------------------------------------ lanes on crystal columns
+// Encoder and decoder give a lane two neighbouring crystal columns of a block:
+// np = ceil(X / 2) lanes a block, nsub = 32 / np blocks side by side in a warp.
+struct Lanes {
+    int np, nsub;
+    __host__ __device__ explicit Lanes(int X) : np((X + 1) / 2), nsub(32 / np < 16 ? 32 / np : 16) {}
 };
 
 // Bit k of byte j of word m -> bit m of byte j of word k (8 x 8 per byte).
@@ -554,6 +85,565 @@ __device__ __forceinline__ void swap_bits8(uint32_t (&p)[8])
     }
 }
 
+// ------------------------------------------------------------------ encoder
+// One pass over the pool.  A chunk is one round (nsub blocks) for each encoder
+// warp of a CTA.  A warp turns its blocks into words staged in shared memory; the
+// last warp of the chunk publishes the chunk's size.  One CTA, the first to run,
+// reads the published sizes in order, as far as they are there, adds them up and
+// writes each chunk's place over its size.  kEncDepth - 1 chunks later the warps
+// write the staged words out at their place: the places come in order, so that
+// every chunk waits for the slowest one before it, and the depth keeps that wait
+// from the encoders.  Chunks go by ticket, so that whatever a chunk waits for is
+// running or done.  (Two stages, and a warp that waited for one chunk's place
+// before it took the next ticket: 1.33 ms.  Decoupled look-back, every chunk
+// reading its predecessors' words: 1.4 ms with 304 chunks in flight, 2.7 with 760.)
+// The two passes before (block sizes, then words, each reading the pool, and
+// three scan kernels between) took 205 + 543 + 13 us for 12.06 M rows x 54, the
+// second bound by issue: a 32 x 32 transpose across the warp for every four
+// columns.  One pass takes 484 us; without the wait for places it would take 395,
+// bound by issue (ALU pipe 67% busy, 16 warps an SM), and its bytes 276.
+//
+// A lane walks its two columns down the block's 32 rows, two samples to a word.
+// Where a column's samples span at most 127, all its differences fit a byte, and
+// the low bytes give them: four rows' bytes to a word, one bytewise subtraction
+// a word, and the bit swaps of the decoder give the planes of the differences;
+// the sign plane xor the others gives the zigzag planes, whose highest non-zero
+// one is the width.  Where a column of the round is wider (pulses: 3% of the
+// blocks of a dense fill, most of those early in a fill), all take 16-bit
+// differences and the swaps on low and high bytes; differences past 16 bits are
+// done a column at a time by the whole warp.  (Every chunk waits for the slowest
+// before it, so a slow round costs more than its share: with one column at a
+// time for all wide ones the pass took 543 us, with every column of such a round
+// sample by sample 646.)  The words' places within the block are
+// one scan over the lanes.
+constexpr int kEncWarps = 8;
+constexpr int kEncThreads = 32 * kEncWarps;
+constexpr int kEncDepth = 6;  // stages of a warp
+constexpr int kEncRing = 16;  // chunks whose tickets and sizes a CTA remembers: at least 2 kEncDepth + 3
+
+// Shared memory of one encoder warp: its stages, what they hold, a round's rows
+// and their barrier.
+struct EncPlan : Lanes {
+    int cap, inb;  // bytes of a stage, of a round's rows
+    __host__ __device__ explicit EncPlan(int X) : Lanes(X)
+    {
+        cap = (28 * nsub * X + 15) & ~15;  // seven words a column; rounds that do not fit are encoded again into place
+        inb = nsub * 64 * X;
+    }
+    __host__ __device__ size_t rows_at() const { return (size_t)kEncDepth * cap; }
+    __host__ __device__ size_t meta_at() const { return rows_at() + (size_t)inb; }
+    __host__ __device__ size_t bar_at() const { return meta_at() + 4 * (size_t)kEncDepth * (1 + nsub); }
+    __host__ __device__ size_t bytes() const { return ((bar_at() + 15) & ~size_t(15)) + 16; }
+    __host__ __device__ long long chunk_blocks() const { return (long long)kEncWarps * nsub; }
+};
+
+// What the warps of a CTA tell each other.
+struct EncShared {
+    long long tk[kEncRing];               // chunk of the CTA's i-th turn
+    unsigned words[kEncRing][kEncWarps];  // words of each warp's round in it
+    unsigned done[kEncRing];              // warps that have encoded it (counted on from turn to turn)
+    int posted;                           // the last turn whose ticket is known
+    int fail, scans;
+};
+
+constexpr unsigned kAgg = 1, kIncl = 2, kGaveUp = 3;
+
+__device__ __forceinline__ unsigned add_acq_rel_cta(unsigned *p, unsigned v)
+{
+    unsigned old;
+    asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(daq::smem_addr(p)), "r"(v) : "memory");
+    return old;
+}
+__device__ __forceinline__ int ld_acquire_cta(const int *p)
+{
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(daq::smem_addr(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_cta(int *p, int v)
+{
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(daq::smem_addr(p)), "r"(v) : "memory");
+}
+
+// The scanning CTA: turns the published sizes of chunks 0, 1, ... into places.
+// Each round reads the next 2 kEncThreads words and takes those before the first
+// that is not there yet.  Returns the payload's words, -1 when it gave up: the
+// chunks that had not got a place are then told so.
+__device__ long long enc_places(unsigned long long *st, long long n_chunks)
+{
+    __shared__ unsigned s_sum[kEncWarps], s_miss[kEncWarps];
+    __shared__ int s_stop;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    long long done = 0, at = 0;
+    uint64_t t0 = daq::global_ns();
+    if (tid == 0) s_stop = 0;
+    __syncthreads();
+    while (done < n_chunks) {
+        unsigned long long v[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const long long c = done + 2 * tid + j;
+            v[j] = c < n_chunks ? daq::ld_relaxed_u64(st + c) : 0ull;
+        }
+        if ((v[0] & 3u) == kGaveUp || (v[1] & 3u) == kGaveUp) s_stop = 1;
+        const unsigned a = (v[0] & 3u) ? (unsigned)(v[0] >> 2) : 0u, b = (v[1] & 3u) ? (unsigned)(v[1] >> 2) : 0u;
+        const unsigned miss = __reduce_min_sync(kFull, !(v[0] & 3u) ? 2u * tid : !(v[1] & 3u) ? 2u * tid + 1 : 2u * kEncThreads);
+        unsigned incl = a + b;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(kFull, incl, d);
+            if (lane >= d) incl += y;
+        }
+        if (lane == 31) s_sum[warp] = incl;
+        if (lane == 0) s_miss[warp] = miss;
+        __syncthreads();
+        unsigned first = 2 * kEncThreads, ahead = 0;
+        for (int w = 0; w < kEncWarps; ++w) {
+            first = min(first, s_miss[w]);
+            if (w < warp) ahead += s_sum[w];
+        }
+        const uint64_t now = daq::global_ns();
+        if (first > 0) t0 = now;
+        if (tid == 0 && now - t0 > kWaitNs) s_stop = 1;
+        // words before this thread's pair; of them only those before `first` count, and every pair before it is whole
+        const long long mine = at + ahead + incl - a - b;
+        if (2 * tid < (int)first) daq::st_relaxed_u64(st + done + 2 * tid, ((unsigned long long)mine << 2) | kIncl);
+        if (2 * tid + 1 < (int)first)
+            daq::st_relaxed_u64(st + done + 2 * tid + 1, ((unsigned long long)(mine + a) << 2) | kIncl);
+        __shared__ long long s_next;
+        if (first > 0 && (unsigned)tid == (first - 1) / 2) s_next = mine + a + ((first & 1) ? 0u : b);
+        __syncthreads();
+        if (s_stop) {
+            for (long long c = done + tid; c < n_chunks; c += kEncThreads) daq::st_relaxed_u64(st + c, kGaveUp);
+            return -1;
+        }
+        if (first > 0) at = s_next;
+        done += first;
+        __syncthreads();
+    }
+    return at;
+}
+
+// Zigzag code of this lane's row of a column (pitch X; the warp, lanes on rows).
+__device__ __forceinline__ uint32_t row_code(const int16_t *col, int X, int lane)
+{
+    const int32_t v = col[lane * X];
+    const int32_t prev = __shfl_up_sync(kFull, v, 1);
+    return lane ? zigzag(v - prev) : 0u;
+}
+
+// a - b in every byte, modulo 256.
+__device__ __forceinline__ uint32_t sub8x4(uint32_t a, uint32_t b)
+{
+    return ((a | 0x80808080u) - (b & 0x7f7f7f7fu)) ^ ((a ^ ~b) & 0x80808080u);
+}
+
+// The zigzag planes of one column from its samples' low bytes (word k, byte j =
+// row 8j + k), in place; returns the width.  All differences fit a byte.
+__device__ __forceinline__ int byte_planes(uint32_t (&p)[8])
+{
+    const uint32_t first = __byte_perm(p[7], p[0], 0x2104);  // rows -1 (row 0 itself), 7, 15, 23
+#pragma unroll
+    for (int k = 7; k > 0; --k) p[k] = sub8x4(p[k], p[k - 1]);
+    p[0] = sub8x4(p[0], first);
+    swap_bits8(p);
+    const uint32_t sign = p[7];
+#pragma unroll
+    for (int k = 7; k > 0; --k) p[k] = p[k - 1] ^ sign;
+    p[0] = sign;
+    int w = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w = p[k] ? k + 1 : w;
+    return w;
+}
+
+// Per 16-bit half, modulo 2^16: v - p (no borrow crosses the halves).
+__device__ __forceinline__ uint32_t sub16x2(uint32_t v, uint32_t p)
+{
+    return ((v | 0x80008000u) - (p & 0x7fff7fffu)) ^ ((v ^ ~p) & 0x80008000u);
+}
+
+// The zigzag planes 0..15 (lo, hi) of one column from the low and high bytes of
+// its differences, in place; returns the width.  All differences fit 16 bits.
+__device__ __forceinline__ int word_planes(uint32_t (&lo)[8], uint32_t (&hi)[8])
+{
+    swap_bits8(lo);
+    swap_bits8(hi);
+    const uint32_t sign = hi[7];
+#pragma unroll
+    for (int k = 7; k > 0; --k) hi[k] = hi[k - 1] ^ sign;
+    hi[0] = lo[7] ^ sign;
+#pragma unroll
+    for (int k = 7; k > 0; --k) lo[k] = lo[k - 1] ^ sign;
+    lo[0] = sign;
+    int w = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w = lo[k] ? k + 1 : w;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w = hi[k] ? k + 9 : w;
+    return w;
+}
+
+// Encode `blocks` <= nsub blocks side by side from the rows at `in` (block pitch
+// 32 X): what a lane has of them.
+template <bool kEven> struct Round {
+    int sub, pr;       // the lane's block and its pair of columns in it
+    bool mine, two;    // the lane has columns, has two
+    const int16_t *col;
+    int X;
+    __device__ __forceinline__ Round(const EncPlan &pl, int X_, const int16_t *in, int blocks, int lane)
+        : sub(lane / pl.np), pr(lane - sub * pl.np), mine(sub < blocks), two(mine && 2 * pr + 1 < X_),
+          col(in + (mine ? sub * 32 * X_ + 2 * pr : 0)), X(X_)
+    {
+    }
+    __device__ __forceinline__ uint32_t row(int r) const  // both samples of row r
+    {
+        if (kEven) return *reinterpret_cast<const uint32_t *>(col + r * X);
+        return (uint32_t)(uint16_t)col[r * X] | (two ? (uint32_t)(uint16_t)col[r * X + 1] << 16 : 0u);
+    }
+    // the lane's words, their place in the round (returned) and the round's
+    // total; `before`: the words ahead of the lane's block
+    __device__ __forceinline__ int place(const EncPlan &pl, int w0, int w1, int lane, int &total, int &before) const
+    {
+        const int words = mine ? 1 + w0 + (two ? 1 + w1 : 0) : 0;
+        int incl = words;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(kFull, incl, d);
+            if (lane >= d) incl += y;
+        }
+        total = __shfl_sync(kFull, incl, 31);
+        before = __shfl_sync(kFull, incl - words, mine ? sub * pl.np : 0);
+        return incl - words;
+    }
+};
+
+// The head word and planes 0 .. 7 of a column at word o; words at or past `room`
+// are dropped.
+__device__ __forceinline__ void store_column(uint32_t *dst, int o, int room, uint32_t first, int w, const uint32_t (&p)[8])
+{
+    if (o < room) dst[o] = first | ((uint32_t)w << 16);
+    const int n = min(w, room - o - 1);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (k < n) dst[o + 1 + k] = p[k];
+}
+
+// A round with a column that is not narrow.  A function of its own: with both
+// forms in one body the narrow one ran 2.3x slower.  Returns the words of the
+// round and those ahead of the lane's block.
+template <bool kEven>
+__device__ __noinline__ int2 encode_wide_round(int X, const int16_t *in, int blocks, uint32_t *dst, int fit, int room)
+{
+    const int lane = threadIdx.x & 31;
+    const EncPlan pl(X);
+    const Round<kEven> R(pl, X, in, blocks, lane);
+    uint32_t p0[8], p1[8], h0[8], h1[8], mx = R.row(0), mn = mx;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        uint32_t d[4];  // differences of rows k, k + 8, ..., both columns
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t v = R.row(8 * j + k);
+            d[j] = 8 * j + k ? sub16x2(v, R.row(8 * j + k - 1)) : 0u;
+            mx = __vmaxs2(mx, v);
+            mn = __vmins2(mn, v);
+        }
+        const uint32_t t = __byte_perm(d[0], d[1], 0x6240), u = __byte_perm(d[2], d[3], 0x6240);
+        const uint32_t th = __byte_perm(d[0], d[1], 0x7351), uh = __byte_perm(d[2], d[3], 0x7351);
+        p0[k] = __byte_perm(t, u, 0x5410);
+        p1[k] = __byte_perm(t, u, 0x7632);
+        h0[k] = __byte_perm(th, uh, 0x5410);
+        h1[k] = __byte_perm(th, uh, 0x7632);
+    }
+    int w0 = word_planes(p0, h0), w1 = word_planes(p1, h1);
+    // columns with differences past 16 bits, one at a time by the whole warp
+    const bool past0 = R.mine && (int)(int16_t)(mx & 0xffffu) - (int)(int16_t)(mn & 0xffffu) > 32767;
+    const bool past1 = R.two && ((int)mx >> 16) - ((int)mn >> 16) > 32767;
+    const unsigned m0 = __ballot_sync(kFull, past0), m1 = __ballot_sync(kFull, past1);
+    const int at = (int)(R.col - in);
+    auto widths = [&](unsigned m, int second, int &w) {
+        for (; m; m &= m - 1u) {
+            const int owner = __ffs(m) - 1;
+            const int v = 32 - __clz(__reduce_or_sync(kFull, row_code(in + __shfl_sync(kFull, at, owner) + second, X, lane)));
+            if (lane == owner) w = v;
+        }
+    };
+    widths(m0, 0, w0);
+    widths(m1, 1, w1);
+    int total, before;
+    const int o0 = R.place(pl, w0, w1, lane, total, before), o1 = o0 + 1 + w0;
+    if (total > fit) return make_int2(total, before);
+    const uint32_t v0 = R.row(0);
+    auto upper = [&](int o, int w, const uint32_t (&h)[8]) {  // planes 8 .. 15
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (k + 8 < min(w, room - o - 1)) dst[o + 9 + k] = h[k];
+    };
+    if (R.mine) {
+        store_column(dst, o0, room, v0 & 0xffffu, w0, p0);
+        upper(o0, w0, h0);
+    }
+    if (R.two) {
+        store_column(dst, o1, room, v0 >> 16, w1, p1);
+        upper(o1, w1, h1);
+    }
+    __syncwarp();
+    auto planes = [&](unsigned m, int second, int w_own, int o_own) {  // over what was stored: lane k stores plane k
+        for (; m; m &= m - 1u) {
+            const int owner = __ffs(m) - 1;
+            const uint32_t z = row_code(in + __shfl_sync(kFull, at, owner) + second, X, lane);
+            const int w = __shfl_sync(kFull, w_own, owner), o = __shfl_sync(kFull, o_own, owner) + 1;
+            uint32_t plane = 0;
+            for (int k = 0; k < w; ++k) {
+                const uint32_t bits = __ballot_sync(kFull, (z >> k) & 1u);
+                if (lane == k) plane = bits;
+            }
+            if (lane < w && o + lane < room) dst[o + lane] = plane;
+        }
+    };
+    planes(m0, 0, w0, o0);
+    planes(m1, 1, w1, o1);
+    return make_int2(total, before);
+}
+
+// Encode a round.  The words go to dst (the first block's first word) when all of
+// them fit `fit` words; words at or past `room` are dropped.  Returns the words of
+// the round; `before` gets those ahead of the lane's block.
+template <bool kEven>
+__device__ __forceinline__ int encode_round(const EncPlan &pl, int X, const int16_t *in, int blocks, uint32_t *dst, int fit,
+                                            int room, int lane, int &before)
+{
+    const Round<kEven> R(pl, X, in, blocks, lane);
+    uint32_t p0[8], p1[8];
+    const uint32_t v0 = R.row(0);
+    uint32_t mx = v0, mn = v0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const uint32_t a = R.row(k), b = R.row(k + 8), c = R.row(k + 16), d = R.row(k + 24);
+        mx = __vimax3_s16x2(__vimax3_s16x2(mx, a, b), c, d);
+        mn = __vimin3_s16x2(__vimin3_s16x2(mn, a, b), c, d);
+        const uint32_t t = __byte_perm(a, b, 0x6240), u = __byte_perm(c, d, 0x6240);  // low bytes of both columns
+        p0[k] = __byte_perm(t, u, 0x5410);
+        p1[k] = __byte_perm(t, u, 0x7632);
+    }
+    const int span0 = (int)(int16_t)(mx & 0xffffu) - (int)(int16_t)(mn & 0xffffu);
+    const int span1 = ((int)mx >> 16) - ((int)mn >> 16);
+    if (__any_sync(kFull, R.mine && max(span0, span1) > 127)) {
+        const int2 r = encode_wide_round<kEven>(X, in, blocks, dst, fit, room);
+        before = r.y;
+        return r.x;
+    }
+    const int w0 = byte_planes(p0), w1 = byte_planes(p1);
+    int total;
+    const int o0 = R.place(pl, w0, w1, lane, total, before);
+    if (total > fit) return total;
+    if (R.mine) store_column(dst, o0, room, v0 & 0xffffu, w0, p0);
+    if (R.two) store_column(dst, o0 + 1 + w0, room, v0 >> 16, w1, p1);
+    return total;
+}
+
+// status: one word a chunk, zeroed, then the ticket and the role counter.  A row
+// copy that does not land, or a wait that runs out, makes the chunk and every
+// later one give up: *out_bytes is -1.
+template <bool kEven>
+__global__ void __launch_bounds__(kEncThreads, 2) pack_kernel(const int16_t *pool, long long rows, int X, long long nb,
+                                                              unsigned long long *status, long long n_chunks,
+                                                              unsigned char *out, long long cap, long long *out_bytes)
+{
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ EncShared sh;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const EncPlan pl(X);
+    uint32_t *out32 = reinterpret_cast<uint32_t *>(out);
+    unsigned long long *table = reinterpret_cast<unsigned long long *>(out + 16);
+    const long long head = 16 + 8 * (nb + 1);
+    unsigned long long *tickets = status + n_chunks;
+    auto entry = [&](long long b, long long words) {  // the offset of block b
+        if (16 + 8 * b + 8 <= cap) table[b] = 4ull * (unsigned long long)words;
+    };
+    if (threadIdx.x == 0) {
+        sh.scans = atomicAdd(tickets + 1, 1ull) == 0ull;  // the first CTA to run
+        sh.fail = 0;
+        sh.posted = 0;
+        for (int k = 0; k < kEncRing; ++k) sh.done[k] = 0;
+        if (!sh.scans) sh.tk[0] = (long long)atomicAdd(tickets, 1ull);
+    }
+    __syncthreads();
+    if (sh.scans) {
+        if (threadIdx.x == 0 && cap >= 16) {
+            out32[0] = kMagic;
+            out32[1] = (uint32_t)X;
+            reinterpret_cast<unsigned long long *>(out)[1] = (unsigned long long)rows;
+        }
+        const long long words = enc_places(status, n_chunks);
+        if (threadIdx.x == 0) {
+            if (words >= 0) entry(nb, words);
+            *out_bytes = words >= 0 ? head + 4 * words : -1ll;
+        }
+        return;
+    }
+
+    unsigned char *base = dsm + warp * pl.bytes();
+    auto stage = [&](int k) { return reinterpret_cast<uint32_t *>(base + k * pl.cap); };
+    int16_t *in = reinterpret_cast<int16_t *>(base + pl.rows_at());
+    unsigned *meta = reinterpret_cast<unsigned *>(base + pl.meta_at());  // per stage: words, then those ahead of each block
+    uint64_t *bar = reinterpret_cast<uint64_t *>(base + pl.bytes() - 16);
+    if (lane == 0) {
+        daq::mbar_init(bar, 1);
+        daq::fence_mbar_init();
+    }
+    __syncwarp();
+    const long long nfull = rows / 32, cb = pl.chunk_blocks();
+    const int sub = lane / pl.np;
+    auto block_of = [&](long long c) { return c * cb + (long long)warp * pl.nsub; };  // this warp's first block of chunk c
+    auto blocks_at = [&](long long b) { return (int)max(0ll, min((long long)pl.nsub, nb - b)); };
+    auto gave_up = [&] { *reinterpret_cast<volatile int *>(&sh.fail) = 1; };
+    bool copying = false;  // a copy of the next round's rows is in flight
+    uint32_t phase = 0;    // that its wait expects
+    auto start_rows = [&](long long c) {
+        const long long b = block_of(c);
+        const int n = blocks_at(b);
+        if (c >= n_chunks || n == 0 || b + n > nfull) return;  // the last, shorter block comes in by plain loads
+        copying = true;
+        if (lane == 0) {
+            daq::fence_proxy_async_smem();
+            daq::mbar_arrive_expect_tx(bar, (uint32_t)(n * 64 * X));
+            daq::bulk_g2s(in, pool + 32 * b * X, (uint32_t)(n * 64 * X), bar);
+        }
+    };
+    auto fits = [&](int j) { return 4 * (int)meta[(j % kEncDepth) * (1 + pl.nsub)] <= pl.cap; };  // turn j's words
+    // write turn j out; v: what was read of its place (lane 0)
+    auto finish = [&](int j, unsigned long long v) {
+        const long long c = sh.tk[j % kEncRing];
+        long long at = -1;
+        if (lane == 0) {
+            const uint64_t t0 = daq::global_ns();
+            while ((v & 3u) < kIncl && !*reinterpret_cast<volatile int *>(&sh.fail)) {
+                v = daq::ld_relaxed_u64(status + c);
+                if (daq::global_ns() - t0 > 2 * kWaitNs) gave_up();
+            }
+            if ((v & 3u) == kIncl) at = (long long)(v >> 2);
+            else gave_up();
+            (void)add_acq_rel_cta(&sh.done[j % kEncRing], 0u);  // the warps' words have been seen
+        }
+        at = __shfl_sync(kFull, at, 0);
+        if (at < 0) return;
+        for (int w = 0; w < warp; ++w) at += sh.words[j % kEncRing][w];
+        const unsigned *m = meta + (j % kEncDepth) * (1 + pl.nsub);
+        const int words = (int)m[0];
+        const long long b = block_of(c);
+        const int n = blocks_at(b);
+        if (lane == sub * pl.np && sub < n) entry(b + sub, at + m[1 + sub]);
+        const int room = (int)(max(0ll, min(cap - (head + 4 * at), 1ll << 30)) >> 2);
+        uint32_t *dst = out32 + (head >> 2) + at;
+        if (fits(j)) {
+            const uint32_t *src = stage(j % kEncDepth);
+            const int last = min(words, room);
+#pragma unroll 4
+            for (int k = lane; k < last; k += 32) dst[k] = src[k];
+        } else {
+            // did not fit the stage: encoded again, into its place (no rows are in flight)
+            for (int k = 0; k < n; ++k) load_block(pool, rows, X, b + k, in + k * 32 * X, lane);
+            int before;
+            encode_round<kEven>(pl, X, in, n, dst, 1 << 30, room, lane, before);
+        }
+        __syncwarp();
+    };
+    long long c = sh.tk[0];
+    start_rows(c);
+    int i = 0;
+    for (; c < n_chunks; ++i) {
+        unsigned long long ticket = 0, place = 0;
+        if (threadIdx.x == 0) ticket = atomicAdd(tickets, 1ull);  // of turn i + 1, used once this one is encoded
+        const int j = i - (kEncDepth - 1);
+        if (lane == 0 && j >= 0) place = daq::ld_relaxed_u64(status + sh.tk[j % kEncRing]);
+        const long long b = block_of(c);
+        const int n = blocks_at(b);
+        if (copying) {
+            const bool ok = daq::mbar_wait_bounded(bar, phase, kWaitNs);
+            phase ^= 1u;
+            copying = false;
+            if (__any_sync(kFull, !ok) && lane == 0) gave_up();
+        } else {
+            for (int k = 0; k < n; ++k) load_block(pool, rows, X, b + k, in + k * 32 * X, lane);
+        }
+        int before;
+        const int fit = pl.cap / 4;
+        const int words = encode_round<kEven>(pl, X, in, n, stage(i % kEncDepth), fit, fit, lane, before);
+        unsigned *m = meta + (i % kEncDepth) * (1 + pl.nsub);
+        if (lane == sub * pl.np && sub < pl.nsub) m[1 + sub] = (unsigned)before;
+        if (lane == 0) {
+            m[0] = (unsigned)words;
+            sh.words[i % kEncRing][warp] = (unsigned)words;
+            if (warp == 0) {
+                sh.tk[(i + 1) % kEncRing] = (long long)ticket;
+                st_release_cta(&sh.posted, i + 1);
+            }
+            const unsigned turn = (unsigned)kEncWarps * (unsigned)(i / kEncRing + 1);
+            if (add_acq_rel_cta(&sh.done[i % kEncRing], 1u) + 1u == turn) {  // the chunk's last warp
+                unsigned total = 0;
+                for (int w = 0; w < kEncWarps; ++w) total += sh.words[i % kEncRing][w];
+                const bool bad = *reinterpret_cast<volatile int *>(&sh.fail);
+                daq::st_relaxed_u64(status + c, bad ? (unsigned long long)kGaveUp : ((unsigned long long)total << 2) | kAgg);
+            }
+            const uint64_t t0 = daq::global_ns();
+            while (ld_acquire_cta(&sh.posted) < i + 1)  // warp 0 has encoded this turn
+                if (daq::global_ns() - t0 > 3 * kWaitNs) {
+                    gave_up();
+                    break;
+                }
+        }
+        __syncwarp();
+        const long long next = sh.tk[(i + 1) % kEncRing];
+        const bool again = j >= 0 && !fits(j);  // turn j needs the row buffer
+        if (!again) start_rows(next);
+        if (j >= 0) finish(j, place);
+        if (again) start_rows(next);
+        c = next;
+    }
+    for (int j = max(0, i - (kEncDepth - 1)); j < i; ++j) finish(j, 0ull);
+}
+
+// ------------------------------------------------------------------ decoder
+// Bound by instruction issue and, at the end, by HBM (61% of its rate).  Lanes
+// own crystal columns, two neighbouring ones each (np = ceil(X / 2) lanes a
+// block, nsub = 32 / np blocks side by side), so a column's bit planes become
+// samples inside one lane: seven three-input operations undo the zigzag on the
+// planes, three stages of bit swaps among eight words (48 operations) turn
+// them into 32 signed bytes (word k, byte j = row 8j + k), and one dp4a a row
+// takes its byte and adds it to the running sample.  A row is one 32-bit store
+// of the lane's two samples; whole blocks leave by bulk copy.  With lanes on
+// rows a column took a 32 x 32 transpose and a prefix sum across the warp, 49
+// instructions a column and warp against 12 here: 12.06 M rows x 54 decoded in
+// 1.19 ms, now 0.34 (the call 1275 -> 383 us).
+// Where the columns' words begin is known only by walking their head words, a
+// chain of X shared-memory loads, so a warp stages the payload of up to G = 4
+// consecutive blocks (16-byte asynchronous copies) and G lanes walk them at
+// once; more would cost occupancy (10 KB a warp, 20 warps an SM).  The next
+// group's payload is brought into L2 while this one is decoded (390 -> 383
+// us).  Undoing the zigzag on bytes after the swaps, copying rows out with
+// 16-byte stores and checking every head word in the walk took 502 us.
+// Columns wider than 8 bits (pulses: 2% of the blocks of a dense fill hold some)
+// are then done again by the whole warp, lanes on rows.
+constexpr int kDecWarps = 4;
+constexpr int kDecThreads = 32 * kDecWarps;
+
+// Lanes, blocks and shared memory of one warp, by the crystal count.
+struct DecPlan : Lanes {
+    int G, cap;  // blocks staged at once, bytes of staged payload
+    __host__ __device__ explicit DecPlan(int X) : Lanes(X)
+    {
+        G = nsub >= 4 ? nsub : nsub == 3 ? 6 : 4;
+        // planes of 6.5 bits a column; one block of the widest columns always fits
+        const int want = G * X * 30, least = X * 72;
+        cap = ((want > least ? want : least) + 15) & ~15;
+    }
+    __host__ __device__ size_t pos_at() const { return (size_t)cap + 32; }  // staged words begin at any 4-byte phase
+    __host__ __device__ size_t out_at(int X) const { return (pos_at() + 2 * (size_t)G * X + 15) & ~size_t(15); }
+    __host__ __device__ size_t bytes(int X) const { return out_at(X) + (size_t)nsub * 64 * X; }
+};
+
 // The differences of a column of width w <= 8 as signed bytes: its zigzag
 // codes' sign plane is plane 0, and bit k of the difference is plane k + 1
 // xor the sign, so seven three-input operations on the planes undo the zigzag
@@ -565,32 +655,6 @@ __device__ __forceinline__ void column_steps(const uint32_t *h, int w, uint32_t 
     for (int k = 0; k < 7; ++k) p[k] = (h[2 + k] & (uint32_t)((k + 1 - w) >> 31)) ^ sign;
     p[7] = sign;
     swap_bits8(p);
-}
-
-// Planes [k0, k0 + 8) of a column as bytes; planes past its width are zero.
-__device__ __forceinline__ void column_bytes(const uint32_t *h, int w, int k0, uint32_t (&p)[8])
-{
-#pragma unroll
-    for (int k = 0; k < 8; ++k) p[k] = k0 + k < w ? h[1 + k0 + k] : 0u;
-    swap_bits8(p);
-}
-
-// One column of any width (<= 17) into every row of the block at out (pitch X).
-__device__ __noinline__ void decode_wide_column(const uint32_t *h, int X, int16_t *out)
-{
-    const int w = (int)(h[0] >> 16);
-    uint32_t lo[8], hi[8];
-    column_bytes(h, w, 0, lo);
-    column_bytes(h, w, 8, hi);
-    const uint32_t top = w > 16 ? h[17] : 0u;
-    int32_t v = (int16_t)(h[0] & 0xffffu);
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        const int k = r & 7, j = r >> 3;
-        const uint32_t z = ((lo[k] >> (8 * j)) & 0xffu) | (((hi[k] >> (8 * j)) & 0xffu) << 8) | (((top >> r) & 1u) << 16);
-        if (r) v += unzigzag(z);
-        out[r * X] = (int16_t)v;
-    }
 }
 
 template <bool kEven>
@@ -625,6 +689,27 @@ __global__ void __launch_bounds__(kDecThreads, 5) unpack_kernel(const unsigned c
     auto bulk_read_done = [&] {
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         __syncwarp();
+    };
+    // columns wider than 8 bits (owner lanes m, head words at h, first rows at o),
+    // one at a time by the whole warp, lanes on rows
+    auto wide_columns = [&](unsigned m, const uint32_t *h, int16_t *o) {
+        const uint32_t *words = reinterpret_cast<const uint32_t *>(base);
+        const int hw = (int)(h - words), oe = (int)(o - out);
+        for (; m; m &= m - 1u) {
+            const int owner = __ffs(m) - 1;
+            const uint32_t *hc = words + __shfl_sync(kFull, hw, owner);
+            int16_t *oc = out + __shfl_sync(kFull, oe, owner);
+            const int w = (int)(hc[0] >> 16);
+            uint32_t z = 0;
+            for (int k = 0; k < w; ++k) z |= ((hc[1 + k] >> lane) & 1u) << k;
+            int32_t d = lane ? unzigzag(z) : 0;
+#pragma unroll
+            for (int s = 1; s < 32; s <<= 1) {
+                const int32_t y = __shfl_up_sync(kFull, d, s);
+                if (lane >= s) d += y;
+            }
+            oc[lane * X] = (int16_t)((int32_t)(int16_t)(hc[0] & 0xffffu) + d);
+        }
     };
     auto offset_of = [&](long long b) { return lane <= pl.G && b + lane <= nb ? offs[b + lane] : ~0ull; };
     unsigned long long next_off = b0 < nb ? offset_of(b0) : 0ull;
@@ -725,33 +810,30 @@ __global__ void __launch_bounds__(kDecThreads, 5) unpack_kernel(const unsigned c
                 const uint32_t v0 = mine ? h0[0] : 0u, v1 = two ? h1[0] : 0u;
                 const int w0 = (int)(v0 >> 16), w1 = (int)(v1 >> 16);
                 int16_t *o = out + (sub < pl.nsub ? sub : 0) * 32 * X + x0;
-                if (!__any_sync(kFull, max(w0, w1) > 8)) {
-                    uint32_t p0[8], p1[8];
-                    column_steps(h0, w0, p0);
-                    column_steps(h1, w1, p1);
-                    bulk_read_done();
-                    int32_t a0 = (int32_t)v0, a1 = (int32_t)v1;  // the low halves count
-                    if (mine) {
+                uint32_t p0[8], p1[8];
+                column_steps(h0, w0, p0);
+                column_steps(h1, w1, p1);
+                bulk_read_done();
+                int32_t a0 = (int32_t)v0, a1 = (int32_t)v1;  // the low halves count
+                if (mine) {
 #pragma unroll
-                        for (int q = 0; q < 32; ++q) {
-                            const int k = q & 7, j = q >> 3;
-                            if (q) {
-                                a0 = __dp4a((int)p0[k], 1 << (8 * j), a0);
-                                a1 = __dp4a((int)p1[k], 1 << (8 * j), a1);
-                            }
-                            if (kEven) {
-                                *reinterpret_cast<uint32_t *>(o + q * X) = __byte_perm((uint32_t)a0, (uint32_t)a1, 0x5410);
-                            } else {
-                                o[q * X] = (int16_t)a0;
-                                if (two) o[q * X + 1] = (int16_t)a1;
-                            }
+                    for (int q = 0; q < 32; ++q) {
+                        const int k = q & 7, j = q >> 3;
+                        if (q) {
+                            a0 = __dp4a((int)p0[k], 1 << (8 * j), a0);
+                            a1 = __dp4a((int)p1[k], 1 << (8 * j), a1);
+                        }
+                        if (kEven) {
+                            *reinterpret_cast<uint32_t *>(o + q * X) = __byte_perm((uint32_t)a0, (uint32_t)a1, 0x5410);
+                        } else {
+                            o[q * X] = (int16_t)a0;
+                            if (two) o[q * X + 1] = (int16_t)a1;
                         }
                     }
-                } else {
-                    bulk_read_done();
-                    if (mine) decode_wide_column(h0, X, o);
-                    if (two) decode_wide_column(h1, X, o + 1);
                 }
+                __syncwarp();
+                wide_columns(__ballot_sync(kFull, w0 > 8), h0, o);
+                wide_columns(__ballot_sync(kFull, w1 > 8), h1, o + 1);
                 __syncwarp();
                 // rows of the good blocks to the pool: a bulk copy per whole block
                 const bool whole = 32 * (b0 + g0 + r + pl.nsub) <= rows;
@@ -786,8 +868,8 @@ __global__ void __launch_bounds__(kDecThreads, 5) unpack_kernel(const unsigned c
 // needs (smem_max; a later call must never lower it), and the resident count
 // is found once per (kernel slot, device, n_xtal) and kept.
 constexpr int kGridDevices = 16;
-int g_resident[5][kGridDevices][kMaxX + 1] = {};  // CTAs resident per GPU, 0 = not known yet
-bool g_limit_set[5][kGridDevices] = {};
+int g_resident[4][kGridDevices][kMaxX + 1] = {};  // CTAs resident per GPU, 0 = not known yet
+bool g_limit_set[4][kGridDevices] = {};
 
 template <typename K>
 int pipelined_grid(int slot, K kernel, int X, int threads, size_t smem, size_t smem_max, long long want)
@@ -811,23 +893,9 @@ int pipelined_grid(int slot, K kernel, int X, int threads, size_t smem, size_t s
     return (int)std::max<long long>(1, std::min<long long>(want, (long long)resident));
 }
 
-struct PackWs {
-    size_t sizes, offs, chunk, widths, err, total;
-};
-
-PackWs pack_ws(long long nb, int X)
-{
-    auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
-    PackWs w;
-    w.sizes = 0;
-    w.offs = up(8 * (size_t)std::max<long long>(nb, 1));
-    w.chunk = up(w.offs + 8 * (size_t)(nb + 1));
-    const long long n_chunks = (nb + kScanChunk - 1) / kScanChunk;
-    w.widths = up(w.chunk + 8 * (size_t)(n_chunks + 1));
-    w.err = up(w.widths + (size_t)std::max<long long>(nb, 1) * (size_t)X);
-    w.total = up(w.err + sizeof(int));
-    return w;
-}
+// Workspace: one status word per chunk, then the ticket and the role counter.
+long long enc_chunks(long long nb, int X) { return (nb + EncPlan(X).chunk_blocks() - 1) / EncPlan(X).chunk_blocks(); }
+size_t pack_ws(long long nb, int X) { return (8 * (size_t)(enc_chunks(nb, X) + 2) + 255) & ~size_t(255); }
 
 }  // namespace daq_pack
 
@@ -845,7 +913,7 @@ int64_t daq_pack_bound(int64_t rows, int n_xtal)
 int daq_pack_workspace_size(int64_t rows, int n_xtal, size_t *bytes)
 {
     if (!bytes || rows < 0 || n_xtal < 1 || n_xtal > kMaxX) return DAQ_EINVAL;
-    *bytes = pack_ws((rows + 31) / 32, n_xtal).total;
+    *bytes = pack_ws((rows + 31) / 32, n_xtal);
     return DAQ_OK;
 }
 
@@ -858,36 +926,17 @@ int daq_pack_pool(const int16_t *pool, int64_t rows, int n_xtal, void *out, int6
         (reinterpret_cast<uintptr_t>(pool) & 15))
         return DAQ_EINVAL;
     const long long nb = (rows + 31) / 32;
-    const PackWs w = pack_ws(nb, n_xtal);
-    if (!workspace || workspace_bytes < w.total || (reinterpret_cast<uintptr_t>(workspace) & 15)) return DAQ_EINVAL;
+    if (!workspace || workspace_bytes < pack_ws(nb, n_xtal) || (reinterpret_cast<uintptr_t>(workspace) & 15)) return DAQ_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    unsigned char *ws = static_cast<unsigned char *>(workspace);
-    auto *sizes = reinterpret_cast<unsigned long long *>(ws + w.sizes);
-    auto *offs = reinterpret_cast<unsigned long long *>(ws + w.offs);
-    auto *chunk = reinterpret_cast<unsigned long long *>(ws + w.chunk);
-    auto *widths = reinterpret_cast<uint8_t *>(ws + w.widths);
-    auto *perr = reinterpret_cast<int *>(ws + w.err);
-    unsigned char *o = static_cast<unsigned char *>(out);
-    const long long n_apply = nb / kScanChunk + 1;  // blocks covering entries 0..nb
-    const size_t smem_size = kWarps * BlockPipe::bytes(n_xtal, 0);
-    const size_t smem_write = kWarps * BlockPipe::bytes(n_xtal, kMaxX);
-    const bool pairs = (n_xtal % 2) == 0;
-    const auto write_kernel = pairs ? pack_write_kernel<true> : pack_write_kernel<false>;
-    const size_t max_size = kWarps * BlockPipe::bytes(kMaxX, 0), max_write = kWarps * BlockPipe::bytes(kMaxX, kMaxX);
-    const long long want = (nb + kWarps - 1) / kWarps;
-    const int g_size = nb > 0 ? pipelined_grid(0, pack_size_kernel, n_xtal, kThreads, smem_size, max_size, want) : 1;
-    const int g_write = pipelined_grid(pairs ? 1 : 2, write_kernel, n_xtal, kThreads, smem_write, max_write,
-                                       std::max<long long>(want, 1));
-    if (g_size < 1 || g_write < 1) return DAQ_ECUDA;
-    if (cudaMemsetAsync(perr, 0, sizeof(int), s) != cudaSuccess) return DAQ_ECUDA;
-    if (nb > 0) pack_size_kernel<<<g_size, kThreads, smem_size, s>>>(pool, rows, n_xtal, nb, sizes, widths, perr);
-    if (nb > 0) scan_reduce_kernel<<<(unsigned)((nb + kScanChunk - 1) / kScanChunk), kThreads, 0, s>>>(sizes, nb, chunk);
-    else if (cudaMemsetAsync(chunk, 0, 8, s) != cudaSuccess) return DAQ_ECUDA;
-    scan_top_kernel<<<1, 1024, 0, s>>>(chunk, nb > 0 ? (nb + kScanChunk - 1) / kScanChunk : 0);
-    scan_apply_kernel<<<(unsigned)n_apply, kThreads, 0, s>>>(sizes, nb, chunk, offs, o, out_cap,
-                                                             reinterpret_cast<long long *>(out_bytes), perr);
-    write_kernel<<<g_write, kThreads, smem_write, s>>>(pool, rows, n_xtal, nb, offs, widths, o, out_cap,
-                                                       reinterpret_cast<long long *>(out_bytes));
+    const long long n_chunks = enc_chunks(nb, n_xtal);
+    const bool even = (n_xtal % 2) == 0;
+    const auto kernel = even ? pack_kernel<true> : pack_kernel<false>;
+    const size_t smem = kEncWarps * EncPlan(n_xtal).bytes(), most = kEncWarps * EncPlan(kMaxX).bytes();
+    const int grid = pipelined_grid(even ? 0 : 1, kernel, n_xtal, kEncThreads, smem, most, n_chunks + 1);
+    if (grid < 1) return DAQ_ECUDA;
+    if (cudaMemsetAsync(workspace, 0, 8 * (size_t)(n_chunks + 2), s) != cudaSuccess) return DAQ_ECUDA;
+    kernel<<<grid, kEncThreads, smem, s>>>(pool, rows, n_xtal, nb, static_cast<unsigned long long *>(workspace), n_chunks,
+                                           static_cast<unsigned char *>(out), out_cap, reinterpret_cast<long long *>(out_bytes));
     return cudaGetLastError() == cudaSuccess ? DAQ_OK : DAQ_ECUDA;
 }
 
@@ -905,7 +954,7 @@ int daq_unpack_pool(const void *in, int64_t in_bytes, int64_t rows, int n_xtal, 
     const auto kernel = even ? unpack_kernel<true> : unpack_kernel<false>;
     const DecPlan pl(n_xtal);
     const size_t most = kDecWarps * DecPlan(kMaxX).bytes(kMaxX);
-    const int grid = pipelined_grid(even ? 3 : 4, kernel, n_xtal, kDecThreads, kDecWarps * pl.bytes(n_xtal), most,
+    const int grid = pipelined_grid(even ? 2 : 3, kernel, n_xtal, kDecThreads, kDecWarps * pl.bytes(n_xtal), most,
                                     (std::max<long long>(nb, 1) + kDecWarps * pl.G - 1) / (kDecWarps * pl.G));
     if (grid < 1) return DAQ_ECUDA;
     kernel<<<grid, kDecThreads, kDecWarps * pl.bytes(n_xtal), s>>>(static_cast<const unsigned char *>(in), in_bytes, rows,

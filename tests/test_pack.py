@@ -192,3 +192,25 @@ def test_decoder_follows_any_valid_offsets(env, X, kind):
     bad[16 + 8 * (nb + 1) + off + 2] = 18
     with pytest.raises(daq.DaqError):
         daq.unpack_pool(torch.from_numpy(bad).cuda(), rows, X)
+
+
+@pytest.mark.gpu
+def test_many_chunks_of_every_kind(env):
+    """Enough blocks that every CTA of the encoder takes many turns, with
+    stretches of noise, of steps past a byte, and of full-range samples whose
+    words fit no stage and are encoded again into place."""
+    torch, daq, oracle = env["torch"], env["daq"], env["oracle"]
+    rng = np.random.default_rng(77)
+    rows, X = 900_007, 33
+    pool = 1800 + rng.integers(-9, 10, size=(rows, X))
+    for k in range(0, rows, 40_000):
+        n = int(rng.integers(1, 6_000))
+        pool[k: k + n] += rng.integers(-600, 600, size=pool[k: k + n].shape) * (rng.random(pool[k: k + n].shape) < 0.05)
+        pool[k + 10_000: k + 10_000 + n] = rng.integers(-32768, 32768, size=pool[k + 10_000: k + 10_000 + n].shape)
+    pool = pool.astype(np.int16)
+    want = oracle.pack(pool)
+    dev = torch.from_numpy(pool).cuda()
+    for _ in range(2):
+        got, n = daq.pack_pool(dev)
+        assert n == want.size and np.array_equal(got.cpu().numpy(), want)
+    assert np.array_equal(daq.unpack_pool(got, rows, X).cpu().numpy(), pool)
