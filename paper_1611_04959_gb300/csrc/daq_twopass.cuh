@@ -212,7 +212,7 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
 
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
-            mbar_init(full + s, kRows ? 33 * NSW : 1);
+            mbar_init(full + s, kRows ? 33 * NSW : 2);  // the copy's thread twice: bytes, tile record
             mbar_init(sums + s, NSW);
             mbar_init(mdone + s, 1);
         }
@@ -228,12 +228,16 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
     constexpr int kSumThreads = 32 * NSW;
 
     uint32_t pend = 0, pend_par = 0;  // thread 0: slots with a load issued, parity of its phase
+    int ptot_next = 0, ptot_slot = -1;  // thread 0: pedestal sum on its way, and its slot
     auto start_load = [&](long long tile, int s) {  // thread 0
         if (kFused &&
             !wait_counter_ge(a, compacted_ctr(a), tile > a.lag_tiles ? (unsigned long long)(tile - a.lag_tiles) : 0ull))
             return;  // gave up (the flag is set): the sum warps stop at this slot
         TileInfo &T = tinfo[s];
-        decode_tile<TW>(a, tile, T, plan.fts, plan.lens);
+        // the pedestal sum is loaded once the copy is on its way and stored by
+        // finish_load a tile later: its load from global memory would stand
+        // before every refill of a slot
+        decode_tile<TW>(a, tile, T, plan.fts, plan.lens, false);
         trace_stamp(a, tile, 0);
         trace_value(a, tile, 10, sm_id());
         trace_value(a, tile, 11, TW);
@@ -247,6 +251,14 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
             }
         }
         trace_stamp(a, tile, 1);
+        ptot_next = a.ptot[(long long)T.f * a.n_calo + T.c];
+        ptot_slot = s;
+    };
+    auto finish_load = [&] {  // thread 0: the record of the last load started is whole
+        if (ptot_slot < 0) return;
+        tinfo[ptot_slot].ptot = ptot_next;
+        if (a.use_tma) mbar_arrive(full + ptot_slot);
+        ptot_slot = -1;
     };
     auto start_rows = [&](long long j, int s) {  // kRows: every sum warp
         const TileInfo T = tinfo[j % (2 * NS)];
@@ -269,8 +281,12 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
         if (kRows || tid == 0)
             for (int k = 0; k < NS; ++k)
                 if (first + k * G < total) {
-                    if constexpr (kRows) start_rows(k, k);
-                    else start_load(first + k * G, k);
+                    if constexpr (kRows) {
+                        start_rows(k, k);
+                    } else {
+                        start_load(first + k * G, k);
+                        finish_load();
+                    }
                 }
         for (long long j = 0;; ++j) {
             const long long tile = first + j * G;
@@ -300,8 +316,12 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
             }
             const uint32_t slot_s = smem_addr(slot);
             for (int it = warp; it < n_steps; it += NSW)
-                sum_pass_step<kRows>(a, T, slot_s, it, NBT, abyte0 + 128 * s, blocksum0 + NBT * s,
-                                     sarr0 + (a.need_sarr ? TW * s : 0), nullptr, lane);
+                if constexpr (kRows)
+                    sum_pass_step<true>(a, T, slot_s, it, NBT, abyte0 + 128 * s, blocksum0 + NBT * s,
+                                        sarr0 + (a.need_sarr ? TW * s : 0), nullptr, lane);
+                else
+                    sum_step_quarters(a, T, slot_s, it, NBT, abyte0 + 128 * s, blocksum0 + NBT * s,
+                                      sarr0 + (a.need_sarr ? TW * s : 0), lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(sums + s);
             if constexpr (kRows) {
@@ -315,6 +335,7 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
                 }
             } else if (tid == 0) {
                 trace_stamp(a, T.tile, 3);
+                finish_load();  // of tile j + NS - 1
                 // slot s takes tile j + NS once every sum warp is done with tile j
                 if (tile + NS * G < total) {
                     if (mbar_wait_bounded(sums + s, par, kWaitLimitNs)) {
