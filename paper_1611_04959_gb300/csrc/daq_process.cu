@@ -200,13 +200,22 @@ __global__ void __launch_bounds__(kThreads) daq_prepare_kernel(KArgs a, int tw)
                     const int x = x0 + k * kWarps;
                     if (x >= a.n_xtal) break;
                     const uint32_t w[4] = {(uint32_t)v[k].x, (uint32_t)v[k].y, (uint32_t)v[k].z, (uint32_t)v[k].w};
-                    long long sum = 0;
+                    int sum = 0;  // 256 samples at most: 32 bits hold it
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const int16_t val = (int16_t)((w[j >> 1] >> (16 * (j & 1))) & 0xffffu);
                         if (8 * lane + j < n) sum += val;
                     }
-                    finish(x, sum);
+                    sum = __reduce_add_sync(kFull, sum);
+                    const int m = (int)n;
+                    int p = 0;
+                    if (m > 0) {
+                        const int num = sum + m / 2;
+                        p = num / m;
+                        if (p * m > num) --p;  // rounded down
+                    }
+                    if (lane == 0 && a.ped_out && !(a.flags & DAQ_SKIP_ISLANDS)) a.ped_out[cf * a.n_xtal + x] = p;
+                    ptot_part += p;
                 }
             }
         } else {

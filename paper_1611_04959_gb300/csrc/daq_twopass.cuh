@@ -85,8 +85,39 @@ struct PlanView {
 __device__ __forceinline__ PlanView cache_plan(const KArgs &a, long long *fts_s, int32_t *lens_s, int tid, int nthr)
 {
     if (a.n_fills > kPlanSmem) return PlanView{a.fill_tile_start, a.lens};
-    for (int f = tid; f <= a.n_fills; f += nthr) fts_s[f] = a.fill_tile_start[f];
-    for (int f = tid; f < a.n_fills; f += nthr) lens_s[f] = a.lens[f];
+    for (int f = tid; f <= a.n_fills; f += nthr) fts_s[f] = __ldcg(a.fill_tile_start + f);
+    for (int f = tid; f < a.n_fills; f += nthr) lens_s[f] = __ldcg(a.lens + f);
+    return PlanView{fts_s, lens_s};
+}
+
+// The same plan worked out by warp 0 from the call's own inputs, for a kernel that
+// starts before the prepare kernel has written it (at most kPlanSmem fills; the
+// caller syncs).
+template <int TW>
+__device__ __forceinline__ PlanView own_plan(const KArgs &a, long long *fts_s, int32_t *lens_s, int tid)
+{
+    static_assert(kPlanSmem == 64, "two fills a lane");
+    if (tid < 32) {
+        long long len[2], tiles[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int f = 2 * tid + i;
+            len[i] = f < a.n_fills ? (a.fill_len ? (long long)__ldcg(a.fill_len + f) : a.n_samples) : 0;
+            len[i] = len[i] < 0 ? 0 : (len[i] > a.n_samples ? a.n_samples : len[i]);
+            tiles[i] = (len[i] + TW - 1) / TW * a.n_calo;
+        }
+        long long total;
+        const long long before = warp_excl_scan_add<long long>(tiles[0] + tiles[1], tid, total);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int f = 2 * tid + i;
+            if (f < a.n_fills) {
+                lens_s[f] = (int32_t)len[i];
+                fts_s[f] = before + (i ? tiles[0] : 0);
+            }
+        }
+        if (tid == 0) fts_s[a.n_fills] = total;
+    }
     return PlanView{fts_s, lens_s};
 }
 
@@ -208,7 +239,14 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
     uint64_t *full = bars, *sums = bars + NS, *mdone = bars + 2 * NS;
 
     for (int i = tid; i < 32 * NS; i += kThr) reinterpret_cast<uint32_t *>(abyte0)[i] = 0u;
-    const PlanView plan = cache_plan(a, fts_s, lens_s, tid, kThr);
+    // The first loads go out before the prepare kernel is waited for: they need the
+    // samples and the plan, not its pedestals.  (This, the compact pass's first
+    // load before the scan is waited for, the scan's ticket before the counts and
+    // 32-bit pedestal sums: 663 -> 657 us a full fill, 107 -> 98 us for two short
+    // calorimeters, waited for.)
+    const bool early = !kFused && a.n_fills <= kPlanSmem;
+    if (!kFused && !early) pdl_wait();
+    const PlanView plan = early ? own_plan<TW>(a, fts_s, lens_s, tid) : cache_plan(a, fts_s, lens_s, tid, kThr);
 
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
@@ -220,15 +258,16 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
     }
     __syncthreads();
     const long long total = plan.fts[a.n_fills];
-    if constexpr (kRows) {
-        if (tid < 2 * NS && first + tid * G < total) decode_tile<TW>(a, first + tid * G, tinfo[tid], plan.fts, plan.lens);
-        __syncthreads();
-    }
     const int n_steps = (a.ew + 63) / 64;
     constexpr int kSumThreads = 32 * NSW;
 
     uint32_t pend = 0, pend_par = 0;  // thread 0: slots with a load issued, parity of its phase
     int ptot_next = 0, ptot_slot = -1;  // thread 0: pedestal sum on its way, and its slot
+    auto load_ptot = [&](int s) {  // thread 0: of the tile whose load was started into slot s
+        ptot_next = a.ptot[(long long)tinfo[s].f * a.n_calo + tinfo[s].c];
+        ptot_slot = s;
+    };
+    bool ptot_ready = kFused;  // the prepare kernel has been waited for
     auto start_load = [&](long long tile, int s) {  // thread 0
         if (kFused &&
             !wait_counter_ge(a, compacted_ctr(a), tile > a.lag_tiles ? (unsigned long long)(tile - a.lag_tiles) : 0ull))
@@ -251,8 +290,7 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
             }
         }
         trace_stamp(a, tile, 1);
-        ptot_next = a.ptot[(long long)T.f * a.n_calo + T.c];
-        ptot_slot = s;
+        if (ptot_ready) load_ptot(s);
     };
     auto finish_load = [&] {  // thread 0: the record of the last load started is whole
         if (ptot_slot < 0) return;
@@ -277,17 +315,37 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
         return kFused ? warp_wait_abortable(a, bar, parity) : warp_wait(bar, parity);
     };
 
-    if (warp < NSW) {
-        if (kRows || tid == 0)
-            for (int k = 0; k < NS; ++k)
-                if (first + k * G < total) {
-                    if constexpr (kRows) {
-                        start_rows(k, k);
-                    } else {
-                        start_load(first + k * G, k);
-                        finish_load();
-                    }
+    if constexpr (kRows) {
+        if (tid < 2 * NS && first + tid * G < total)
+            decode_tile<TW>(a, first + tid * G, tinfo[tid], plan.fts, plan.lens, false);
+        __syncthreads();
+    }
+    if (warp < NSW && (kRows || tid == 0))
+        for (int k = 0; k < NS; ++k)
+            if (first + k * G < total) {
+                if constexpr (kRows) {
+                    start_rows(k, k);
+                } else {
+                    start_load(first + k * G, k);
+                    finish_load();
                 }
+            }
+    if (early) pdl_wait();       // the prepare kernel's pedestals and resets
+    if (!kFused) pdl_trigger();  // the scan may be scheduled as CTAs finish
+    if constexpr (kRows) {
+        if (tid < 2 * NS && first + tid * G < total)
+            tinfo[tid].ptot = a.ptot[(long long)tinfo[tid].f * a.n_calo + tinfo[tid].c];
+        __syncthreads();
+    } else if (!kFused && tid == 0) {
+        ptot_ready = true;
+        for (int k = 0; k < NS; ++k)
+            if (first + k * G < total) {
+                load_ptot(k);
+                finish_load();
+            }
+    }
+
+    if (warp < NSW) {
         for (long long j = 0;; ++j) {
             const long long tile = first + j * G;
             if (tile >= total) break;
@@ -431,8 +489,6 @@ template <int TW, int NS, bool HF, bool ROWS>
 __global__ void __launch_bounds__(count_threads<NS>(), NS == 2 ? 2 : 1) daq_count_kernel(const __grid_constant__ KArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    pdl_wait();     // the prepare kernel's plan, pedestals and resets
-    pdl_trigger();  // the scan may be scheduled as CTAs finish
     count_role<TW, false, NS, HF, ROWS>(a, smem, blockIdx.x, gridDim.x);
 }
 
@@ -555,8 +611,8 @@ template <int TW> __device__ TileRec complete_tile(const KArgs &a, long long j)
 template <int TW, bool HF>
 __global__ void __launch_bounds__(kScanThreads) daq_scan_kernel(const __grid_constant__ KArgs a)
 {
-    pdl_wait();  // every tile's record
-    pdl_trigger();
+    // the prepare kernel's plan and reset are there (the count kernel waits for it
+    // before it lets this one start): the ticket is taken while counts finish
     __shared__ Agg warp_tot[kScanThreads / 32];
     __shared__ Agg s_incl[kScanThreads];
     __shared__ Agg s_prefix;
@@ -564,8 +620,10 @@ __global__ void __launch_bounds__(kScanThreads) daq_scan_kernel(const __grid_con
     if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(a.scan_ticket, 1u);
     __syncthreads();
     const long long chunk = s_chunk;
-    const long long total = a.fill_tile_start[a.n_fills];
+    const long long total = __ldcg(a.fill_tile_start + a.n_fills);
     const long long chunk0 = chunk * kScanChunk;
+    pdl_wait();  // every tile's record
+    pdl_trigger();
     if (chunk0 >= total) return;  // grids are sized for the largest tile count
     const long long base = chunk0 + (long long)threadIdx.x * kScanPer;
     TileRec *recs = reinterpret_cast<TileRec *>(a.recs);
@@ -764,7 +822,7 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
     // marks (box k holds columns [k boxw, (k + 1) boxw)); the single-launch
     // form's records may not be published yet: all.
     auto flags_of = [&](long long tile) -> uint32_t {
-        return (kFused || tile >= total) ? ~0u : (uint32_t)recs[tile].flags;
+        return (kFused || tile >= total) ? ~0u : (uint32_t)__ldcg(&recs[tile].flags);
     };
     auto boxes_of = [&](uint32_t flags) -> uint32_t {
         if (flags == ~0u) return all_boxes;
@@ -861,21 +919,34 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
 
     uint32_t phase_bit = 0;
     bool store_pending = false;
-    bool load_pending = false;  // thread 32 (single-launch form): a load issued that no thread has waited for
+    bool load_pending = false;  // thread 32: a load issued that no thread has waited for
     uint32_t nMt = 0, nfl2 = 0;
     int nm2 = 1;  // kSparse, lane 0 of warp 0: marked samples of the next tile + G
     TileRec nr{0, 0, 0, 0};
     TileExcl ne{0, 0, 0};
     int in_ok = 1;
+    // the first tile's load goes out before the scan is waited for: it needs the
+    // plan and (unless the scan completes them) the count pass's records
     if (first < total) {
+        const uint32_t boxes = boxes_of(a.halo_free ? ~0u : flags_of(first));
         if constexpr (kRows) {
             if (tid == 0) decode_tile<TW>(a, first, tinfo_r[0], plan.fts, plan.lens, false);
             __syncthreads();
-            start_rows(boxes_of(flags_of(first)));
+            start_rows(boxes);
         } else if (tid == 32) {
-            start_load(first, boxes_of(flags_of(first)));
-            load_pending = kFused;
+            start_load(first, boxes);
+            load_pending = a.use_tma;
         }
+    }
+    if constexpr (!kFused) {
+        pdl_wait();        // every tile's prefix
+        if (aborted(a)) {  // the scan gave up: its prefixes are incomplete
+            if (kRows) row_load_wait();
+            else if (tid == 32 && load_pending) mbar_wait_bounded(bar, 0, kWaitLimitNs);
+            return;
+        }
+    }
+    if (first < total) {
         if (warp == 0) in_ok = load_inputs(first, nMt, nr, ne, nm2, nfl2) ? 1 : 0;
     }
     for (long long tile = first; tile < total;) {
@@ -1004,8 +1075,6 @@ __device__ __forceinline__ void compact_role(const KArgs &a, unsigned char *smem
 template <int TW, bool kSparse, bool ROWS>
 __global__ void __launch_bounds__(256, 2) daq_compact_kernel(const __grid_constant__ KArgs a)
 {
-    pdl_wait();                // every tile's prefix
-    if (aborted(a)) return;    // the scan gave up: its prefixes are incomplete
     extern __shared__ __align__(128) unsigned char smem[];
     compact_role<TW, false, kSparse, ROWS>(a, smem, blockIdx.x, gridDim.x);
 }
