@@ -260,6 +260,13 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
                       const daq_params *params, const daq_islands *islands_out, int64_t *qhist_inout);
 
 /*
+ * Wait for everything queued on `stream` so far, copy a call's counts[4] to host
+ * memory and return the call's status (as DAQ_SYNC does, for callers that want the
+ * counts too): one wait for both.  DAQ_EINVAL for a null pointer.
+ */
+int daq_read_counts(const int64_t *counts, int64_t *counts_host, void *stream);
+
+/*
  * Host buffers of daq_process_fills_host (the end-to-end form).
  *   samples_host   host int16[n_fills][n_calo][n_xtal][n_samples]; page-locked
  *                  memory gives full copy bandwidth.

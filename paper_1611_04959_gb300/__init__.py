@@ -134,6 +134,8 @@ def lib():
             L.daq_process_fills_host.restype = i32
             L.daq_trace_tiles.argtypes = [i32, i32, i64, i32, ctypes.POINTER(DaqParams)]
             L.daq_trace_tiles.restype = i64
+            L.daq_read_counts.argtypes = [vp, vp, vp]
+            L.daq_read_counts.restype = i32
             L.daq_status_from_counts.argtypes = [vp]
             L.daq_status_from_counts.restype = i32
             L.daq_strerror.argtypes = [i32]
@@ -233,6 +235,12 @@ def daq_process_fills(samples_ptr: int, n_calo: int, n_xtal: int, n_samples: int
                       params: DaqParams, islands: DaqIslands, qhist_ptr: int | None) -> int:
     return int(lib().daq_process_fills(samples_ptr, n_calo, n_xtal, n_samples, n_fills, ctypes.byref(params),
                                        ctypes.byref(islands), qhist_ptr))
+
+
+def daq_read_counts(counts_ptr: int, counts_host: np.ndarray, stream=None) -> int:
+    """Wait for `stream`, read counts[4] into counts_host and return the call's status."""
+    return int(lib().daq_read_counts(counts_ptr, counts_host.ctypes.data,
+                                     None if stream is None else int(stream.cuda_stream)))
 
 
 def daq_process_fills_static(samples_ptr: int, n_calo: int, n_xtal: int, n_samples: int, n_fills: int,
@@ -349,7 +357,7 @@ def pack_pool(pool, rows: int | None = None, stream=None, out=None, workspace=No
     need = daq_pack_workspace_size(rows, X)
     if workspace is None or workspace.numel() < need:
         workspace = torch.empty(need, dtype=torch.uint8, device=dev)
-    nbytes = torch.zeros(1, dtype=torch.int64, device=dev)
+    nbytes = torch.empty(1, dtype=torch.int64, device=dev)   # always written by the call
     stream = torch.cuda.current_stream(dev) if stream is None else stream
     rc = daq_pack_pool(pool.data_ptr(), rows, X, out.data_ptr(), out.numel(), nbytes.data_ptr(), workspace.data_ptr(),
                        workspace.numel(), stream.cuda_stream)
@@ -364,7 +372,7 @@ def unpack_pool(packed, rows: int, n_xtal: int, stream=None):
     import torch
     dev = packed.device
     out = torch.empty((max(1, rows), n_xtal), dtype=torch.int16, device=dev)
-    err = torch.zeros(1, dtype=torch.int32, device=dev)
+    err = torch.empty(1, dtype=torch.int32, device=dev)      # the call clears it
     stream = torch.cuda.current_stream(dev) if stream is None else stream
     rc = daq_unpack_pool(packed.data_ptr(), packed.numel(), rows, n_xtal, out.data_ptr(), err.data_ptr(),
                          stream.cuda_stream)
@@ -461,14 +469,19 @@ def process_fills(samples, threshold=30, pre=8, post=24, ped_samples=100, decim=
         workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=dev)
     p.workspace, p.workspace_bytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
     if sync:
-        p.flags |= DAQ_SYNC
+        p.flags &= ~DAQ_SYNC      # the counts are wanted too: one wait for both
     rc = daq_process_fills(samples.data_ptr(), C, X, N, F, p, outputs.struct(),
                            None if q is None else q.data_ptr())
+    counts = None
+    if sync and rc == DAQ_OK:
+        counts = np.empty(4, np.int64)
+        rc = daq_read_counts(outputs.counts.data_ptr(), counts, stream)
     res = dict(outputs=outputs, q=q, workspace=workspace, status=rc)
     if rc not in (DAQ_OK, DAQ_ECAPACITY) and rc not in allow:
         raise DaqError(rc, "daq_process_fills")
     if sync:
-        counts = outputs.counts.cpu().numpy()
+        if counts is None:        # not queued, with a status the caller allows
+            counts = outputs.counts.cpu().numpy()
         res.update(counts=counts, n_islands=int(counts[0]), n_rows=int(counts[1]))
     return res
 

@@ -159,3 +159,10 @@ def test_no_cpu_fallback_when_library_missing(tmp_path, monkeypatch):
     monkeypatch.setattr(d, "LIB_PATH", str(tmp_path / "libdaq.so"))
     with pytest.raises(RuntimeError, match="not built"):
         d.lib()
+
+
+def test_read_counts_rejects_null_pointers(daq):
+    import numpy as np
+    h = np.zeros(4, np.int64)
+    assert daq.daq_read_counts(None, h) == daq.DAQ_EINVAL
+    assert daq.lib().daq_read_counts(8, None, None) == daq.DAQ_EINVAL
