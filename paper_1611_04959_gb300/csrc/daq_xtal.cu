@@ -77,64 +77,128 @@ __global__ void __launch_bounds__(kThreads) xtal_prepare_kernel(const int16_t *s
     }
 }
 
-// kVec: rows 16-byte aligned (pitch % 8 == 0): 16-byte sample loads, 64-byte Q
-// accesses; otherwise element by element.
-template <bool kVec>
-__global__ void __launch_bounds__(kThreads) xtal_sum_kernel(const int16_t *samples, int n_fills, int n_calo,
-                                                            int n_xtal, int64_t pitch, const int32_t *lens,
-                                                            const int32_t *ped, long long *q)
+__device__ __forceinline__ void load_q(const long long *p, long long (&v)[8], bool wide)
 {
-    const long long chunks = (pitch + 7) / 8;
+    if (wide) {  // 32 bytes an access: every lane takes whole sectors
+#pragma unroll
+        for (int k = 0; k < 8; k += 4)
+            asm volatile("ld.global.v4.s64 {%0, %1, %2, %3}, [%4];"
+                         : "=l"(v[k]), "=l"(v[k + 1]), "=l"(v[k + 2]), "=l"(v[k + 3])
+                         : "l"(p + k)
+                         : "memory");
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+            const longlong2 t = *reinterpret_cast<const longlong2 *>(p + k);
+            v[k] = t.x;
+            v[k + 1] = t.y;
+        }
+    }
+}
+
+__device__ __forceinline__ void store_q(long long *p, const long long (&v)[8], bool wide)
+{
+    if (wide) {
+#pragma unroll
+        for (int k = 0; k < 8; k += 4)
+            asm volatile("st.global.v4.s64 [%0], {%1, %2, %3, %4};" ::"l"(p + k), "l"(v[k]), "l"(v[k + 1]), "l"(v[k + 2]),
+                         "l"(v[k + 3])
+                         : "memory");
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) __stcs(reinterpret_cast<longlong2 *>(p + k), make_longlong2(v[k], v[k + 1]));
+    }
+}
+
+// Bound by HBM: 2 bytes a sample, 16 bytes a cell.  A thread owns 8 consecutive
+// cells of the whole array [n_calo][n_xtal][pitch], whatever the pitch, so that its
+// accumulators are 64-byte aligned and (where one fill's samples are a multiple of
+// 8, or there is one fill) its samples 16-byte aligned; a group of 8 may hold the
+// end of one row and the start of the next.  Accumulators move 32 bytes a lane and
+// access, whole sectors: 24 x 54 x 560,000 cells take 1.94 ms (6.75 TB/s, the copy
+// rate) against 2.17 with accesses of 16 bytes, 64 apart from lane to lane, and
+// 3.03 with lanes on consecutive 16 bytes and 4-byte sample loads.  Groups within a
+// row, taken sample by sample where the pitch is odd, took 1.70 ms for three fills of
+// 24 x 54 x 99,999; these take 0.48.  Four CTAs an SM: at five the 64 registers do
+// not suffice (2.22 ms).
+// kVec: aligned 16-byte sample loads, of kAhead fills at once (two: 721 us for four
+// fills of 140,000 samples against 731 with one and 748 with four, whose registers
+// cost a CTA); wide: q is 32-byte aligned.  I: the index type, 32 bits where the
+// cells allow (one division a group).
+template <bool kVec, int kAhead, typename I>
+__global__ void __launch_bounds__(kThreads, 4) xtal_sum_kernel(const int16_t *samples, int n_fills, int n_calo,
+                                                            int n_xtal, int64_t pitch, const int32_t *lens,
+                                                            const int32_t *ped, long long *q, bool wide)
+{
     const long long n_rows = (long long)n_calo * n_xtal;
-    const long long total = n_rows * chunks;
-    const long long cx_stride = (long long)n_calo * n_xtal * pitch;  // one fill
-    for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < total; i += (long long)gridDim.x * kThreads) {
-        const long long row = i / chunks;
-        const long long t0 = (i - row * chunks) * 8;
+    const long long cells = n_rows * pitch;
+    const long long groups = (cells + 7) / 8;
+    for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < groups; i += (long long)gridDim.x * kThreads) {
+        const long long at = 8 * i;
+        const I row = (I)at / (I)pitch;
+        const long long t0 = at - (long long)row * pitch;
+        const bool full = at + 8 <= cells;
+        const bool one_row = full && t0 + 8 <= pitch;
         long long acc[8];
+        if (full) {  // the accumulators' loads go out before the samples'
+            load_q(q + at, acc, wide);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] = 0;
-        long long *dst = q + row * pitch + t0;
-        const bool vec_q = kVec && t0 + 8 <= pitch;
-        longlong2 o[4];
-        if (vec_q) {  // the accumulators' loads go out before the samples'
-            const longlong2 *d2 = reinterpret_cast<const longlong2 *>(dst);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) o[k] = d2[k];
+            for (int k = 0; k < 8; ++k) acc[k] = at + k < cells ? q[at + k] : 0;
         }
-        for (int f = 0; f < n_fills; ++f) {
-            const long long len = lens[f];
-            if (t0 >= len) continue;
-            const int16_t *src = samples + (long long)f * cx_stride + row * pitch + t0;
-            const long long P = ped[(long long)f * n_rows + row];
-            if (kVec && t0 + 8 <= len) {
-                const int4 v = __ldcs(reinterpret_cast<const int4 *>(src));  // streamed: read once
-                const uint32_t w[4] = {(uint32_t)v.x, (uint32_t)v.y, (uint32_t)v.z, (uint32_t)v.w};
+        for (int f0 = 0; f0 < n_fills; f0 += kAhead) {
+            int4 v[kAhead];
+            if (kVec && full) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    acc[2 * k] += (long long)(int16_t)(w[k] & 0xffffu) - P;
-                    acc[2 * k + 1] += (long long)(int16_t)(w[k] >> 16) - P;
+                for (int u = 0; u < kAhead; ++u)
+                    if (f0 + u < n_fills)
+                        v[u] = __ldcs(reinterpret_cast<const int4 *>(samples + (long long)(f0 + u) * cells + at));  // read once
+            }
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const int f = f0 + u;
+                if (f >= n_fills) break;
+                const long long len = lens[f];
+                const int32_t *P = ped + (long long)f * n_rows + row;
+                if (kVec && one_row && t0 + 8 <= len) {
+                    const int p = P[0];
+                    const uint32_t w[4] = {(uint32_t)v[u].x, (uint32_t)v[u].y, (uint32_t)v[u].z, (uint32_t)v[u].w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {  // a sample less a pedestal fits 32 bits
+                        acc[2 * k] += (int)(int16_t)(w[k] & 0xffffu) - p;
+                        acc[2 * k + 1] += (int)(int16_t)(w[k] >> 16) - p;
+                    }
+                } else if (!one_row || t0 < len) {
+                    // the end of a row, of the fill or of the array
+                    const int16_t *src = samples + (long long)f * cells + at;
+                    long long t = t0;
+                    int r = 0;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        if (at + k < cells && t < len) acc[k] += (int)src[k] - P[r];
+                        if (++t == pitch) {
+                            t = 0;
+                            ++r;
+                        }
+                    }
                 }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (t0 + k < len) acc[k] += (long long)src[k] - P;
             }
         }
-        if (vec_q) {
-            longlong2 *d2 = reinterpret_cast<longlong2 *>(dst);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                o[k].x += acc[2 * k];
-                o[k].y += acc[2 * k + 1];
-                __stcs(d2 + k, o[k]);
-            }
+        if (full) {
+            store_q(q + at, acc, wide);
         } else {
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-                if (t0 + k < pitch) dst[k] += acc[k];
+                if (at + k < cells) q[at + k] = acc[k];
         }
     }
+}
+
+using SumKernel = void (*)(const int16_t *, int, int, int, int64_t, const int32_t *, const int32_t *, long long *, bool);
+template <int kAhead> SumKernel pick(bool vec, bool small)
+{
+    if (vec) return small ? xtal_sum_kernel<true, kAhead, uint32_t> : xtal_sum_kernel<true, kAhead, unsigned long long>;
+    return small ? xtal_sum_kernel<false, kAhead, uint32_t> : xtal_sum_kernel<false, kAhead, unsigned long long>;
 }
 
 int grid_for(long long work)
@@ -182,14 +246,11 @@ int daq_crystal_sum(const int16_t *samples, int n_calo, int n_xtal, int64_t n_sa
         samples, n_fills, n_calo, n_xtal, n_samples, params->fill_len, params->ped_samples, lens, ped, status);
     if (cudaGetLastError() != cudaSuccess) return DAQ_ECUDA;
     if (cells > 0 && n_fills > 0) {
-        const long long work = (long long)n_calo * n_xtal * ((n_samples + 7) / 8);
-        const bool vec = n_samples % 8 == 0 && (reinterpret_cast<uintptr_t>(samples) & 15) == 0;
-        if (vec)
-            xtal_sum_kernel<true><<<grid_for(work), kThreads, 0, s>>>(samples, n_fills, n_calo, n_xtal, n_samples,
-                                                                      lens, ped, reinterpret_cast<long long *>(q_xtal));
-        else
-            xtal_sum_kernel<false><<<grid_for(work), kThreads, 0, s>>>(samples, n_fills, n_calo, n_xtal, n_samples,
-                                                                       lens, ped, reinterpret_cast<long long *>(q_xtal));
+        const bool vec = (cells % 8 == 0 || n_fills == 1) && (reinterpret_cast<uintptr_t>(samples) & 15) == 0;
+        const bool wide = (reinterpret_cast<uintptr_t>(q_xtal) & 31) == 0, small = cells <= (int64_t)0xffffffff;
+        const auto kernel = n_fills == 1 ? pick<1>(vec, small) : pick<2>(vec, small);
+        kernel<<<grid_for((cells + 7) / 8), kThreads, 0, s>>>(samples, n_fills, n_calo, n_xtal, n_samples, lens, ped,
+                                                              reinterpret_cast<long long *>(q_xtal), wide);
         if (cudaGetLastError() != cudaSuccess) return DAQ_ECUDA;
     }
     if (params->flags & DAQ_SYNC) {

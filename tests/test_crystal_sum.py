@@ -86,3 +86,28 @@ def test_full_fill_sampled_rows(env):
     tot = q.sum(dim=(1, 2)).cpu().numpy()
     ref = oracle.process_fills(s, dict(w.params(), threshold=10 ** 9, decim=(560_000,)), n_threads=16)["q"]
     assert np.array_equal(tot, ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("q_shift", [0, 2])
+@pytest.mark.parametrize("F,C,X,N", [(1, 1, 1, 1), (1, 2, 3, 5), (2, 1, 8, 7), (2, 3, 5, 1003), (3, 2, 54, 999),
+                                     (5, 2, 4, 1000), (1, 2, 9, 4001), (4, 1, 54, 2048)])
+def test_groups_that_cross_rows(env, F, C, X, N, shift, q_shift):
+    """A thread's eight cells may hold the end of one row and the start of the
+    next (any pitch), samples and accumulators at every alignment the call takes:
+    rows shorter than a group, uneven fills, an odd tail of the whole array."""
+    torch, daq, oracle = env["torch"], env["daq"], env["oracle"]
+    rng = np.random.default_rng(F * 1000 + N)
+    s = rng.integers(-32768, 32768, size=(F, C, X, N)).astype(np.int16)
+    flat = torch.empty(shift + s.size, dtype=torch.int16, device="cuda")
+    flat[shift:] = torch.from_numpy(s.reshape(-1))
+    x = flat[shift:].view(F, C, X, N)
+    lens = None if N % 2 == 0 else [max(0, N - 3 * f) for f in range(F)]
+    start = rng.integers(-10 ** 12, 10 ** 12, size=(C, X, N))
+    qf = torch.empty(q_shift + start.size, dtype=torch.int64, device="cuda")
+    q = qf[q_shift:].view(C, X, N)
+    q.copy_(torch.from_numpy(start))
+    daq.crystal_sum(x, q=q, fill_len=lens, ped_samples=37)
+    want = oracle.crystal_sum(s, fill_len=lens, ped_samples=37, q=start.copy())
+    assert np.array_equal(q.cpu().numpy(), want)
