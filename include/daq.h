@@ -117,8 +117,19 @@ typedef struct daq_island {
  *                that this form supports and whose shared-memory plan fits
  *                (384 only for the two-pass form, 960 only for the plain
  *                kernel).
- *   grid         0  = two-pass form (count kernel, scan, compact kernel), grids
- *                     from occupancy (default);
+ *   grid         0  = default: the phased form where it pays, else the two-pass
+ *                     form (count kernel, scan, compact kernel), grids from
+ *                     occupancy.  The phased form is one cooperative launch
+ *                     that compacts each tile a few tiles behind its count, so
+ *                     that the second read is from L2: 0.55 ms against 0.66 on
+ *                     24 x 54 x 560,000 samples.  It takes calls that write
+ *                     islands, without DAQ_SPARSE or a trace, of 16-byte
+ *                     aligned rows (n_samples % 8 == 0), an even n_xtal from 40
+ *                     to 56, at most 64 fills, 448-sample tiles, windows of up
+ *                     to some 90 samples, a wait limit of 0 or at least 1 s and
+ *                     14 tiles an SM (2 where the windows are wide: post = 64);
+ *                     a caller confined to some of the SMs gets the two-pass
+ *                     form;
  *                > 0 = two-pass form with exactly this many CTAs per kernel;
  *                -1 = single-pass plain kernel, one CTA per tile;
  *                -2 = single-pass plain kernel, persistent;
@@ -146,7 +157,8 @@ typedef struct daq_island {
  *   events       NULL, or a host array of DAQ_N_EVENTS cudaEvent_t that the call
  *                records on `stream`: [0] start, [1] after the pedestal kernel,
  *                [2] after the count (single-pass: tile) kernel, [3] after the
- *                scan, [4] end (per-kernel timing).
+ *                scan, [4] end (per-kernel timing).  A form of one kernel,
+ *                such as the phased form, records [2], [3] and [4] after it.
  *   trace        NULL, or device uint64[max_tiles][DAQ_TRACE_WORDS] (max_tiles
  *                from daq_trace_tiles()): per-tile %globaltimer stamps of each
  *                stage (profiling only; costs a few stores per tile).
@@ -161,8 +173,8 @@ typedef struct daq_island {
  *                decimation's block of q_calos rows.
  *   wait_limit_ns  limit of each device-side wait on state that other CTAs
  *                publish (0 = 4 s): the look-back over earlier tiles (every
- *                form's scan), and the single-launch form's scanner and lag
- *                waits.  A wait that runs out sets DAQ_DEV_TIMEOUT; every CTA
+ *                form's scan), the single-launch form's scanner and lag
+ *                waits, and the phased form's wait for a chunk's aggregates.  A wait that runs out sets DAQ_DEV_TIMEOUT; every CTA
  *                then stops taking work, waits for its own copies in flight
  *                and exits, and the call returns DAQ_ETIMEOUT with incomplete
  *                outputs.  The next call starts clean.  Waits of a CTA on its

@@ -20,8 +20,10 @@
 //                       decimated partial sums into the int64 Q histograms
 //                       (rows 7-8).
 //
-// Two tile kernels implement the same steps (daq_steps.cuh):
-//   daq_pipe_kernel  the default: one persistent CTA per SM whose warps have
+// The default is the phased form (daq_phase.cuh) or the two-pass form
+// (daq_twopass.cuh).  Two tile kernels implement the same steps in one pass
+// (daq_steps.cuh):
+//   daq_pipe_kernel  one persistent CTA per SM whose warps have
 //                    fixed roles (bulk-load producer, crystal-sum/staging warps,
 //                    window/merge warp, look-back warp, writer warps) handing
 //                    tiles to each other through mbarriers, so loads, scan
@@ -49,6 +51,7 @@
 #include "daq_stream.cuh"
 #include "daq_park.cuh"
 #include "daq_launch.cuh"
+#include "daq_phase.cuh"
 
 namespace daq {
 
@@ -112,6 +115,10 @@ __global__ void __launch_bounds__(kThreads) daq_prepare_kernel(KArgs a, int tw)
         for (long long i = (long long)blockIdx.x * kThreads + tid; i < a.max_tiles; i += (long long)gridDim.x * kThreads)
             rc[i] = make_uint4(0u, 0u, 0u, 0u);
         if (blockIdx.x == 0 && tid < 2) a.fctr[16 * tid] = 0ull;
+    } else if (a.mode == kModePhased) {  // the tiles' published words
+        uint4 *st = reinterpret_cast<uint4 *>(a.status);
+        for (long long i = (long long)blockIdx.x * kThreads + tid; i < (a.max_tiles + 3) / 4; i += (long long)gridDim.x * kThreads)
+            st[i] = make_uint4(0u, 0u, 0u, 0u);
     } else if (a.mode != kModeTwoPass) {  // scan state of the single-pass kernels
         uint4 *st = reinterpret_cast<uint4 *>(a.status);
         const long long n16 = a.max_tiles * (long long)(sizeof(TileStatus) / 16);
@@ -998,6 +1005,47 @@ static int make_plan(int n_calo, int n_xtal, int64_t n_samples, int n_fills, con
     return DAQ_OK;
 }
 
+// Where the phased form takes the place of the two-pass form (us of the two-pass form
+// against it, calls queued, L2 flushed):
+//   tiles     a tile costs it a fixed time on one SM, so it needs enough tiles an SM to
+//             gain by the bytes saved: 51 / 54 at 9.5 tiles an SM, 62 / 61 at 12.8,
+//             77 / 68 at 16.4, 241 / 199 at 66, 665 / 548 at 197.  Where the two-pass
+//             form would leave the halo out and complete marks in its scan
+//             (post = 64), 37 / 27 at 2, 147 / 114 at 33 and 678 / 568 at 197.
+//   crystals  the fixed time counts for more in a smaller tile: 133 / 150 at 12
+//             crystals (8 calorimeters), 526 / 537 at 36, 600 / 550 at 40 (24).
+constexpr int kPhaseMinTiles = 14, kPhaseMinTilesHaloFree = 2;  // an SM
+constexpr int kPhaseMinXtal = 40;
+// a caller's limit on waits below this keeps the two-pass form, which waits less
+constexpr uint64_t kPhaseMinWaitNs = 1000000000ull;
+
+// The phased form's plan in place of a two-pass plan of the same tiles: true if
+// its slots fit, with any halo (a two-pass plan that leaves the halo out to keep two
+// count CTAs per SM takes it in again: a halo is read from L2 here).
+static bool phase_geometry(Plan *pl, int pre, int post, int X)
+{
+    if (pl->mode != kModeTwoPass || pl->tw != kPhaseTile || X < kPhaseMinXtal || X > kPhaseXtal || (X & 1)) return false;
+    Plan r = *pl;
+    plan_geometry(&r, kPhaseTile, pre, post, X);
+    r.mode = kModePhased;
+    r.smem = PhaseSmem<kPhaseTile>(X, r.slot_bytes, r.need_sarr).total;
+    r.smem_b = 0;
+    if (r.nbox_b != 2 || r.boxw_b != kPhaseTile / 2 || r.ew > kMaxExtBits || r.smem > (size_t)kSmemBudget) return false;
+    *pl = r;
+    return true;
+}
+
+// Phased form: one cooperative launch, one CTA per SM.
+static cudaError_t launch_phase(const KArgs &a, const Plan &pl, int sms, cudaStream_t s)
+{
+    static size_t conf[64] = {0};
+    cudaError_t e = ensure_smem(daq_phase_kernel<kPhaseTile>, pl.smem, conf);
+    if (e != cudaSuccess) return e;
+    void *args[] = {const_cast<KArgs *>(&a)};
+    return cudaLaunchCooperativeKernel((const void *)daq_phase_kernel<kPhaseTile>, dim3(std::min(sms, 32 * kPhaseGather)),
+                                       dim3(kPhaseThreads), args, pl.smem, s);
+}
+
 template <int TW> static cudaError_t launch_plain(const KArgs &a, const Plan &pl, int grid, cudaStream_t s)
 {
     static size_t configured[64] = {0};
@@ -1183,12 +1231,39 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     a.srow = stage_row_bytes(n_xtal);
     a.wpr = n_xtal / 2;
     a.wpr_mul = a.wpr > 0 ? (1ull << 32) / (unsigned long long)a.wpr + 1 : 0ull;
-    a.use_tma = 0;
-    if (total > 0 && n_samples % 8 == 0 && (reinterpret_cast<uintptr_t>(samples) & 15) == 0)
-        a.use_tma = encode_tensor_map(&a.tmap, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples, pl.boxw,
+    cudaStream_t s = static_cast<cudaStream_t>(p.stream);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return DAQ_ECUDA;
+    const DeviceInfo di = device_info(dev);
+    if (di.sms <= 0) return DAQ_ECUDA;
+    const bool aligned = total > 0 && n_samples % 8 == 0 && (reinterpret_cast<uintptr_t>(samples) & 15) == 0;
+    auto encode_maps = [&] {
+        a.use_tma = aligned &&
+                    encode_tensor_map(&a.tmap, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples, pl.boxw,
                                       n_xtal) &&
                     encode_tensor_map(&a.tmap_b, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples,
                                       pl.boxw_b, n_xtal);
+    };
+    // The default form is phased where it can be and pays: whole tiles of 448 samples
+    // loaded by boxes, islands written, a plan that fits in shared memory, enough tiles an SM.  Not
+    // with DAQ_SPARSE, whose compact kernel skips what this form would still step
+    // through, nor for a caller's own short limit on waits, which are longer here (a
+    // CTA waits for the slowest of a chunk), nor under a trace.
+    const Plan twopass = pl;
+    if (p.grid == 0 && aligned && !skip_isl && !(p.flags & DAQ_SPARSE) && !p.trace && n_fills <= kPlanSmem &&
+        (p.wait_limit_ns == 0 || p.wait_limit_ns >= kPhaseMinWaitNs) &&
+        pl.max_tiles >= (int64_t)(pl.halo_free ? kPhaseMinTilesHaloFree : kPhaseMinTiles) * di.sms) {
+        if (phase_geometry(&pl, p.pre, p.post, n_xtal) && (int)pl.smem <= di.smem_optin) geometry();
+        else pl = twopass;
+    }
+    encode_maps();
+    auto take_twopass = [&] {
+        pl = twopass;
+        geometry();
+        a.halo_free = pl.halo_free;
+        encode_maps();
+    };
+    if (pl.mode == kModePhased && !a.use_tma) take_twopass();
     if (pl.mode == kModeStream && a.use_tma) {
         PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
         cuuint64_t dims[2] = {(cuuint64_t)n_samples, (cuuint64_t)((int64_t)n_fills * n_calo * n_xtal)};
@@ -1208,11 +1283,7 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
         rc = make_plan(n_calo, n_xtal, n_samples, n_fills, &q, &pl);
         if (rc) return rc;
         geometry();
-        if (total > 0 && n_samples % 8 == 0 && (reinterpret_cast<uintptr_t>(samples) & 15) == 0)
-            a.use_tma = encode_tensor_map(&a.tmap, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples, pl.boxw,
-                                          n_xtal) &&
-                        encode_tensor_map(&a.tmap_b, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples,
-                                          pl.boxw_b, n_xtal);
+        encode_maps();
     }
     if (pl.mode == kModeTwoPass && !a.use_tma && total > 0 && rows_geometry(&pl, n_xtal)) {
         a.use_tma = kLoadRows;
@@ -1247,24 +1318,34 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     a.scan_ticket = reinterpret_cast<unsigned int *>(ws + 384);
     a.trace = reinterpret_cast<unsigned long long *>(p.trace);
 
-    cudaStream_t s = static_cast<cudaStream_t>(p.stream);
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return DAQ_ECUDA;
-    const DeviceInfo di = device_info(dev);
-    if (di.sms <= 0) return DAQ_ECUDA;
     if ((int)pl.smem > di.smem_optin || (int)pl.smem_b > di.smem_optin) return DAQ_EUNSUPPORTED;
 
     cudaEvent_t const *ev = reinterpret_cast<cudaEvent_t const *>(p.events);
     if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return DAQ_ECUDA;
     const long long n_cf = (long long)n_fills * n_calo;
     const int prep_grid = (int)std::max<long long>(1, std::min<long long>(std::max<long long>(n_cf, 1), 4ll * di.sms));
-    daq_prepare_kernel<<<prep_grid, kThreads, 0, s>>>(a, pl.tw);
-    if (cudaError_t e0 = cudaGetLastError()) return cuda_fail(e0);
-    if (ev && cudaEventRecord(ev[1], s) != cudaSuccess) return DAQ_ECUDA;
+    auto prepare = [&]() -> cudaError_t {
+        daq_prepare_kernel<<<prep_grid, kThreads, 0, s>>>(a, pl.tw);
+        if (cudaError_t e0 = cudaGetLastError()) return e0;
+        return ev ? cudaEventRecord(ev[1], s) : cudaSuccess;
+    };
+    if (cudaError_t e0 = prepare()) return cuda_fail(e0);
 
     const int64_t tiles_cap = std::max<int64_t>(1, std::min<int64_t>(pl.max_tiles, INT32_MAX));
-    cudaError_t e;
-    if (pl.mode == kModePark) {
+    cudaError_t e = cudaSuccess;
+    if (pl.mode == kModePhased) {
+        e = launch_phase(a, pl, di.sms, s);
+        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+            // fewer SMs for this caller than the device has: the two-pass form runs on any number
+            cudaGetLastError();
+            take_twopass();
+            e = prepare();
+        }
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (pl.mode == kModePhased) {
+        // launched
+    } else if (pl.mode == kModePark) {
         switch (pl.tw) {
         case 128: e = launch_park<128>(a, pl, di.sms, s); break;
         case 224: e = launch_park<224>(a, pl, di.sms, s); break;

@@ -22,7 +22,7 @@ namespace daq {
 constexpr uint64_t kWaitLimitNs = 4000000000ull;  // bounded device waits (4 s)
 constexpr int kMaxTileWords = 14;                 // marks words of the widest two-pass tile (448 samples)
 // kernels a call may use (daq_params.grid picks one)
-enum : int32_t { kModeTwoPass = 0, kModePlain = 1, kModePipelined = 2, kModeFused = 3, kModeStream = 4, kModePark = 5 };
+enum : int32_t { kModeTwoPass = 0, kModePlain = 1, kModePipelined = 2, kModeFused = 3, kModeStream = 4, kModePark = 5, kModePhased = 6 };
 // daq_params-independent choice of the tile loads: element by element, tensor
 // boxes, or (two-pass form, rows that share no 16-byte alignment) row by row
 enum : int32_t { kLoadPlain = 0, kLoadBoxes = 1, kLoadRows = 2 };
@@ -236,7 +236,7 @@ __device__ __forceinline__ void issue_tile_load(const KArgs &a, const TileInfo &
 {
     const int c0 = (int)(T.t0 - a.hl);
     const int c1 = (int)(((long long)T.f * a.n_calo + T.c) * a.n_xtal);
-    if (a.mode == kModeFused || a.mode == kModeStream) {  // re-read soon by the compaction: keep them in L2
+    if (a.mode == kModeFused || a.mode == kModeStream || a.mode == kModePhased) {  // re-read soon by the compaction: keep them in L2
         const uint64_t pol = l2_policy_evict_last();
         for (int k = 0; k < a.nbox; ++k)
             tma_load_2d_hint(slot + (size_t)k * a.box_stride, &a.tmap, c0 + k * a.boxw, c1, bar, pol);

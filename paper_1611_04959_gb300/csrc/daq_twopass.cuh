@@ -740,7 +740,7 @@ __device__ __forceinline__ void issue_tile_load_b(const KArgs &a, const TileInfo
 {
     const int c0 = (int)T.t0;
     const int c1 = (int)(((long long)T.f * a.n_calo + T.c) * a.n_xtal);
-    const bool last_use = a.mode == kModeFused || a.mode == kModeStream;
+    const bool last_use = a.mode == kModeFused || a.mode == kModeStream || a.mode == kModePhased;
     const uint64_t pol = l2_policy_evict_first();
     for (int k = 0; k < a.nbox_b; ++k) {
         if (!((boxes >> k) & 1u)) continue;
