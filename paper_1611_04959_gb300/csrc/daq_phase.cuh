@@ -6,7 +6,7 @@
 // pool once (6.5 TB/s over both kernels on a full fill).  Here chunk k is one tile for
 // each CTA, one CTA per SM, and a tile is compacted while at most kPhaseAhead chunks
 // of 152 x 48 KB lie between its two reads.  On 24 x 54 x 560,000 samples HBM reads
-// fall from 2.9 to 1.5 GB (the samples are 1.45) and a fill from 657 to 552 us.
+// fall from 2.9 to 1.5 GB (the samples are 1.45) and a fill from 657 to 516 us.
 //
 // Warps of a CTA, handing tiles on through mbarriers:
 //   8 sum        crystal sums, threshold bits and block sums of a tile in one of two
@@ -32,9 +32,10 @@
 // Straight-line code is what the warps' speed hangs on: with one or two warps of a
 // part on a scheduler, instruction fetch is exposed.  The staging stores without a
 // condition (columns that are not marked write to a spare row) and without a case
-// for odd crystal counts took a fill from 652 to 552 us.  Counting by 4 warps: 565;
-// kPhaseAhead 4: 754, 5 to 7: 552; the two jobs in turn by the same warps, two CTAs
-// per SM: 635 at best.
+// for odd crystal counts took a fill from 652 to 552 us, Q bins in 32-bit arithmetic
+// and a kernel for each kind of window (kWin32, kWin96: one form of marks_word each)
+// from there to 516.  At 552: counting by 4 warps 565; kPhaseAhead 4: 754, 5 to 7: 552.
+// The two jobs in turn by the same warps, two CTAs per SM: 635 at best.
 #pragma once
 
 #include "daq_twopass.cuh"
@@ -117,7 +118,7 @@ __device__ __forceinline__ bool phase_vote(bool failed)
     return any != 0;
 }
 
-template <int TW>
+template <int TW, int kWin>
 __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __grid_constant__ KArgs a)
 {
     constexpr int NWT = TW / 32, NBT = TW / 8, R = kPhaseAhead, RI = kPhaseInfo;
@@ -261,7 +262,7 @@ __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __gri
             if (!(ok = warp_wait_abortable(a, sums + b, par2(k)))) break;
             const TileInfo T = tinfo0[k % RI];
             unsigned edges;
-            const uint32_t Mt = tile_marks<TW>(a, T, abyte0 + 128 * b, &edges, lane);
+            const uint32_t Mt = tile_marks<TW, kWin>(a, T, abyte0 + 128 * b, &edges, lane);
             const int nt = (int)(T.t_end - T.t0);
             const Agg agg = words_from_marks<TW>(Mt, edges & 1u, edges >> 1, nt, words_of(k), nullptr, lane);
             const uint32_t steps = marked_steps64<TW>(Mt, lane);

@@ -1006,7 +1006,7 @@ static int make_plan(int n_calo, int n_xtal, int64_t n_samples, int n_fills, con
 }
 
 // Where the phased form takes the place of the two-pass form (us of the two-pass form
-// against it, calls queued, L2 flushed):
+// against it at 552 us a full fill, calls queued, L2 flushed):
 //   tiles     a tile costs it a fixed time on one SM, so it needs enough tiles an SM to
 //             gain by the bytes saved: 51 / 54 at 9.5 tiles an SM, 62 / 61 at 12.8,
 //             77 / 68 at 16.4, 241 / 199 at 66, 665 / 548 at 197.  Where the two-pass
@@ -1024,7 +1024,8 @@ constexpr uint64_t kPhaseMinWaitNs = 1000000000ull;
 // count CTAs per SM takes it in again: a halo is read from L2 here).
 static bool phase_geometry(Plan *pl, int pre, int post, int X)
 {
-    if (pl->mode != kModeTwoPass || pl->tw != kPhaseTile || X < kPhaseMinXtal || X > kPhaseXtal || (X & 1)) return false;
+    if (pl->mode != kModeTwoPass || pl->tw != kPhaseTile || X < kPhaseMinXtal || X > kPhaseXtal || (X & 1) || pre + post > 96)
+        return false;
     Plan r = *pl;
     plan_geometry(&r, kPhaseTile, pre, post, X);
     r.mode = kModePhased;
@@ -1036,14 +1037,15 @@ static bool phase_geometry(Plan *pl, int pre, int post, int X)
 }
 
 // Phased form: one cooperative launch, one CTA per SM.
-static cudaError_t launch_phase(const KArgs &a, const Plan &pl, int sms, cudaStream_t s)
+template <int kWin> static cudaError_t launch_phase(const KArgs &a, const Plan &pl, int sms, cudaStream_t s)
 {
     static size_t conf[64] = {0};
-    cudaError_t e = ensure_smem(daq_phase_kernel<kPhaseTile>, pl.smem, conf);
+    auto kernel = daq_phase_kernel<kPhaseTile, kWin>;
+    cudaError_t e = ensure_smem(kernel, pl.smem, conf);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<KArgs *>(&a)};
-    return cudaLaunchCooperativeKernel((const void *)daq_phase_kernel<kPhaseTile>, dim3(std::min(sms, 32 * kPhaseGather)),
-                                       dim3(kPhaseThreads), args, pl.smem, s);
+    return cudaLaunchCooperativeKernel((const void *)kernel, dim3(std::min(sms, 32 * kPhaseGather)), dim3(kPhaseThreads),
+                                       args, pl.smem, s);
 }
 
 template <int TW> static cudaError_t launch_plain(const KArgs &a, const Plan &pl, int grid, cudaStream_t s)
@@ -1334,7 +1336,7 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     const int64_t tiles_cap = std::max<int64_t>(1, std::min<int64_t>(pl.max_tiles, INT32_MAX));
     cudaError_t e = cudaSuccess;
     if (pl.mode == kModePhased) {
-        e = launch_phase(a, pl, di.sms, s);
+        e = p.pre + p.post <= 32 ? launch_phase<kWin32>(a, pl, di.sms, s) : launch_phase<kWin96>(a, pl, di.sms, s);
         if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
             // fewer SMs for this caller than the device has: the two-pass form runs on any number
             cudaGetLastError();

@@ -541,11 +541,29 @@ __device__ __forceinline__ void sum_step_quarters(const KArgs &a, const TileInfo
 
 // Marks of the 32 extended-tile bits held by this lane: M[i] = OR of A over
 // [i - post, i + pre].  Fast form (post + pre <= 96): the lane gathers the seven
-// threshold words around its own once and widens them in registers.
+// threshold words around its own once and widens them in registers.  A kernel
+// that is compiled for windows of one kind (kWin32: post + pre <= 32, kWin96) holds
+// that form alone.
+constexpr int kWinAny = 0, kWin32 = 1, kWin96 = 2;
+template <int kWin = kWinAny>
 __device__ __forceinline__ uint32_t marks_word(const KArgs &a, uint32_t A, int lane)
 {
     const int L = a.pre + a.post + 1;
-    if (a.pre + a.post <= 96) {
+    if constexpr (kWin == kWin32) {
+        // 64 bits from 32 lane - post on hold all that is needed
+        const uint32_t up = __shfl_up_sync(kFull, A, 1), down = __shfl_down_sync(kFull, A, 1);
+        const unsigned long long w = ((unsigned long long)A << 32) | (lane > 0 ? up : 0u);
+        unsigned long long r = w >> (32 - a.post);
+        if (lane < 31 && a.post < 32) r |= (unsigned long long)down << (32 + a.post);
+        int cov = 1;
+        while (2 * cov <= L) {
+            r |= r >> cov;
+            cov *= 2;
+        }
+        if (cov < L) r |= r >> (L - cov);
+        return (uint32_t)r;
+    }
+    if (kWin == kWin96 || a.pre + a.post <= 96) {
         uint32_t win[8];
 #pragma unroll
         for (int i = 0; i < 7; ++i) {
@@ -707,7 +725,7 @@ __device__ __forceinline__ Agg agg_from_marks(uint32_t Mt, uint32_t m_prev, int 
 // Marks of the tile proper from the threshold bits of the extended tile (one
 // warp): returns this lane's marks word of the tile proper and, through
 // *edges, bit 0 = mark of sample t0 - 1 and bit 1 = mark of sample t0 + TW.
-template <int TW>
+template <int TW, int kWin = kWinAny>
 __device__ __forceinline__ uint32_t tile_marks(const KArgs &a, const TileInfo &T, const uint8_t *abyte,
                                                unsigned *edges, int lane)
 {
@@ -716,7 +734,7 @@ __device__ __forceinline__ uint32_t tile_marks(const KArgs &a, const TileInfo &T
     const int NWE = (a.ew + 31) / 32;
     const long long e0 = T.t0 - HL;
     const uint32_t A = lane < NWE ? reinterpret_cast<const uint32_t *>(abyte)[lane] : 0u;
-    uint32_t Mv = marks_word(a, A, lane);
+    uint32_t Mv = marks_word<kWin>(a, A, lane);
     Mv &= range_mask(32ll * lane, -e0, T.len - e0);  // only samples of [0, len) are marked
     const uint32_t prev_w = __shfl_sync(kFull, Mv, (HL - 1) >> 5);
     const uint32_t next_w = __shfl_sync(kFull, Mv, (HL + TW) >> 5);
@@ -1011,22 +1029,25 @@ __device__ __forceinline__ void write_headers(const KArgs &a, const TileInfo &T,
 __device__ __forceinline__ void q_partial(const KArgs &a, const TileInfo &T, const int32_t *blocksum,
                                           const int32_t *sarr, int gt, int nthr)
 {
+    // 32 bits hold every index (t <= 2^30, k D + D < 2^32); the two 64-bit divisions
+    // cost the phased form 17 us of 560 on a full fill
+    const uint32_t t0 = (uint32_t)T.t0, t_end = (uint32_t)T.t_end;
+    if (t_end <= t0) return;
     for (int d = 0; d < a.n_decim; ++d) {
-        const long long D = a.decim[d];
+        const uint32_t D = (uint32_t)a.decim[d];
         unsigned long long *qrow =
             reinterpret_cast<unsigned long long *>(a.q + a.qoff[d] + (long long)(a.calo_base + T.c) * a.qbins[d]);
-        const long long k_lo = T.t0 / D, k_hi = (T.t_end - 1) / D;
-        for (long long k = k_lo + gt; k <= k_hi; k += nthr) {
-            const long long lo = (k * D > T.t0 ? k * D : T.t0) - T.t0;
-            const long long hi = (k * D + D < T.t_end ? k * D + D : T.t_end) - T.t0;
+        const uint32_t k_lo = t0 / D, k_hi = (t_end - 1u) / D;
+        for (uint32_t k = k_lo + (uint32_t)gt; k <= k_hi; k += (uint32_t)nthr) {
+            const uint32_t lo = max(k * D, t0) - t0, hi = min(k * D + D, t_end) - t0;
             long long sum = 0;
-            if ((D & 7) == 0) {
-                for (long long b = lo >> 3; b < (hi + 7) >> 3; ++b) sum += blocksum[b];
+            if ((D & 7u) == 0u) {
+                for (uint32_t b = lo >> 3; b < (hi + 7u) >> 3; ++b) sum += blocksum[b];
             } else {
-                for (long long t = lo; t < hi; ++t) sum += sarr[t];
+                for (uint32_t t = lo; t < hi; ++t) sum += sarr[t];
             }
             if ((a.flags & DAQ_DEBUG_CHECKS) &&
-                !(k >= 0 && k < a.qbins[d] && a.calo_base + T.c >= 0 && a.calo_base + T.c < a.q_calos)) {
+                !((long long)k < a.qbins[d] && a.calo_base + T.c >= 0 && a.calo_base + T.c < a.q_calos)) {
                 set_status_bit(a, DAQ_DEV_BAD_INDEX);
                 continue;
             }
