@@ -121,13 +121,14 @@ typedef struct daq_island {
  *                     form (count kernel, scan, compact kernel), grids from
  *                     occupancy.  The phased form is one cooperative launch
  *                     that compacts each tile a few tiles behind its count, so
- *                     that the second read is from L2: 0.55 ms against 0.66 on
+ *                     that the second read is from L2: 0.50 ms against 0.66 on
  *                     24 x 54 x 560,000 samples.  It takes calls that write
  *                     islands, without DAQ_SPARSE or a trace, of 16-byte
- *                     aligned rows (n_samples % 8 == 0), an even n_xtal from 40
- *                     to 56, at most 64 fills, 448-sample tiles, windows of up
- *                     to some 90 samples, a wait limit of 0 or at least 1 s and
- *                     14 tiles an SM (2 where the windows are wide: post = 64);
+ *                     aligned rows (n_samples % 8 == 0), an even n_xtal of at
+ *                     most 56, at most 64 fills, 448-sample tiles, windows of
+ *                     up to some 90 samples, a wait limit of 0 or at least 1 s
+ *                     and 14 tiles an SM (2 where the windows are wide:
+ *                     post = 64, 48 crystals);
  *                     a caller confined to some of the SMs gets the two-pass
  *                     form;
  *                > 0 = two-pass form with exactly this many CTAs per kernel;

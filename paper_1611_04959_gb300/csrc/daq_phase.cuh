@@ -6,7 +6,7 @@
 // pool once (6.5 TB/s over both kernels on a full fill).  Here chunk k is one tile for
 // each CTA, one CTA per SM, and a tile is compacted while at most kPhaseAhead chunks
 // of 152 x 48 KB lie between its two reads.  On 24 x 54 x 560,000 samples HBM reads
-// fall from 2.9 to 1.5 GB (the samples are 1.45) and a fill from 657 to 516 us.
+// fall from 2.9 to 1.5 GB (the samples are 1.45) and a fill from 657 to 500 us.
 //
 // Warps of a CTA, handing tiles on through mbarriers:
 //   8 sum        crystal sums, threshold bits and block sums of a tile in one of two
@@ -34,7 +34,8 @@
 // condition (columns that are not marked write to a spare row) and without a case
 // for odd crystal counts took a fill from 652 to 552 us, Q bins in 32-bit arithmetic
 // and a kernel for each kind of window (kWin32, kWin96: one form of marks_word each)
-// from there to 516.  At 552: counting by 4 warps 565; kPhaseAhead 4: 754, 5 to 7: 552.
+// from there to 516, kernels without the code for DAQ_DEBUG_CHECKS and odd decimations
+// (kPlain) to 500.  At 552: counting by 4 warps 565; kPhaseAhead 4: 754, 5 to 7: 552.
 // The two jobs in turn by the same warps, two CTAs per SM: 635 at best.
 #pragma once
 
@@ -118,7 +119,7 @@ __device__ __forceinline__ bool phase_vote(bool failed)
     return any != 0;
 }
 
-template <int TW, int kWin>
+template <int TW, int kWin, bool kPlain>
 __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __grid_constant__ KArgs a)
 {
     constexpr int NWT = TW / 32, NBT = TW / 8, R = kPhaseAhead, RI = kPhaseInfo;
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __gri
             if (!ok) break;
             const TileInfo T = tinfo0[k % RI];
             for (int it = warp; it < n_steps; it += kPhaseSum)
-                sum_step_quarters(a, T, smem_addr(smem + b * L.slot), it, NBT, abyte0 + 128 * b, blocksum0 + NBT * b,
+                sum_step_quarters<kPlain>(a, T, smem_addr(smem + b * L.slot), it, NBT, abyte0 + 128 * b, blocksum0 + NBT * b,
                                   sarr0 + (a.need_sarr ? TW * b : 0), lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(sums + b);
@@ -213,7 +214,10 @@ __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __gri
             // pair of pairs swapped, so that the rows' words, 54 words apart from lane to
             // lane, go to 32 banks.
             uint32_t w[kPhaseXtal], wl0, wl1;
-            {
+            // columns without a marked sample are passed over (24 calorimeters of little
+            // noise: 444 -> 414 us)
+            const bool some = __any_sync(kFull, c < nt && ((W.m[c >> 5] >> (c & 31)) & 3u));
+            if (some) {
                 const int cc = c < nt ? c : 0;
                 const uint32_t at = smem_addr(slot) + (uint32_t)((cc >= kBoxW ? a.box_stride_b : 0) + 2 * (cc >= kBoxW ? cc - kBoxW : cc));
                 const uint32_t at0 = at + flip * 2 * kBoxW, at2 = at - flip * 2 * kBoxW;
@@ -228,7 +232,7 @@ __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __gri
             if ((failed = phase_vote(failed))) break;  // every warp has read the slot
             const long long rb = 2ll * X;
             const int phase = (int)((ex.m * rb) & 15);
-            {
+            if (some) {
                 // a column that is not marked writes to a row of its own, past the slots: the stores need no condition
                 const int wi = c >> 5, bit = c & 31;
                 const uint32_t mw = c < nt ? W.m[wi] : 0u;
@@ -277,7 +281,7 @@ __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __gri
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(marked + k % R);
-            if (!skip_q) q_partial(a, T, blocksum0 + NBT * b, sarr0 + (a.need_sarr ? TW * b : 0), lane, 32);
+            if (!skip_q) q_partial<kPlain>(a, T, blocksum0 + NBT * b, sarr0 + (a.need_sarr ? TW * b : 0), lane, 32);
             __syncwarp();
             if (lane == 0) mbar_arrive(mdone + b);
         }
@@ -335,7 +339,7 @@ __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __gri
             const long long gs = ex.m * rb;
             const int phase = (int)(gs & 15);
             long long ge = gs + (long long)r.m * rb;
-            if ((a.flags & DAQ_DEBUG_CHECKS) && (ex.m < 0 || r.m < 0 || r.m > nt)) {
+            if (!kPlain && (a.flags & DAQ_DEBUG_CHECKS) && (ex.m < 0 || r.m < 0 || r.m > nt)) {
                 if (lane == 0) set_status_bit(a, DAQ_DEV_BAD_INDEX);
                 ge = gs;
             }
@@ -362,7 +366,7 @@ __global__ void __launch_bounds__(kPhaseThreads, 1) daq_phase_kernel(const __gri
                     *reinterpret_cast<uint16_t *>(g + o) = *reinterpret_cast<const uint16_t *>(slot + phase + (o - gs));
                 }
             }
-            write_headers<TW>(a, T, words_of(k), ex, lane);
+            write_headers<TW, kPlain>(a, T, words_of(k), ex, lane);
             __syncwarp();
             if (lane == 0) {
                 bulk_wait_read0();

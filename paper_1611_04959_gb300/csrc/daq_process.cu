@@ -1006,16 +1006,16 @@ static int make_plan(int n_calo, int n_xtal, int64_t n_samples, int n_fills, con
 }
 
 // Where the phased form takes the place of the two-pass form (us of the two-pass form
-// against it at 552 us a full fill, calls queued, L2 flushed):
-//   tiles     a tile costs it a fixed time on one SM, so it needs enough tiles an SM to
-//             gain by the bytes saved: 51 / 54 at 9.5 tiles an SM, 62 / 61 at 12.8,
-//             77 / 68 at 16.4, 241 / 199 at 66, 665 / 548 at 197.  Where the two-pass
-//             form would leave the halo out and complete marks in its scan
-//             (post = 64), 37 / 27 at 2, 147 / 114 at 33 and 678 / 568 at 197.
-//   crystals  the fixed time counts for more in a smaller tile: 133 / 150 at 12
-//             crystals (8 calorimeters), 526 / 537 at 36, 600 / 550 at 40 (24).
-constexpr int kPhaseMinTiles = 14, kPhaseMinTilesHaloFree = 2;  // an SM
-constexpr int kPhaseMinXtal = 40;
+// against it, calls queued, L2 flushed): a tile costs it a fixed time on one SM, so it
+// needs enough tiles an SM to gain by the bytes saved.  54 crystals: 51 / 52 at 9.5
+// tiles an SM, 57 / 56 at 11, 63 / 57 at 12.8, 78 / 65 at 16.4, 663 / 496 at 197.
+// Fewer crystals: 53 / 51 at 16.4 (20 crystals), 374 / 328 (12) and 317 / 273 (4) at 197.
+// Where the two-pass form would leave the halo out and complete the marks in its scan
+// (post = 64): 37 / 27 at 2, 45 / 42 at 5.7 with 54 crystals, 32 / 33 at 4.1 with 36.
+static int phase_min_tiles(const Plan &twopass, int X)  // an SM
+{
+    return twopass.halo_free && X >= 48 ? 2 : 14;
+}
 // a caller's limit on waits below this keeps the two-pass form, which waits less
 constexpr uint64_t kPhaseMinWaitNs = 1000000000ull;
 
@@ -1024,7 +1024,7 @@ constexpr uint64_t kPhaseMinWaitNs = 1000000000ull;
 // count CTAs per SM takes it in again: a halo is read from L2 here).
 static bool phase_geometry(Plan *pl, int pre, int post, int X)
 {
-    if (pl->mode != kModeTwoPass || pl->tw != kPhaseTile || X < kPhaseMinXtal || X > kPhaseXtal || (X & 1) || pre + post > 96)
+    if (pl->mode != kModeTwoPass || pl->tw != kPhaseTile || X > kPhaseXtal || (X & 1) || pre + post > 96)
         return false;
     Plan r = *pl;
     plan_geometry(&r, kPhaseTile, pre, post, X);
@@ -1037,10 +1037,11 @@ static bool phase_geometry(Plan *pl, int pre, int post, int X)
 }
 
 // Phased form: one cooperative launch, one CTA per SM.
-template <int kWin> static cudaError_t launch_phase(const KArgs &a, const Plan &pl, int sms, cudaStream_t s)
+template <int kWin, bool kPlain>
+static cudaError_t launch_phase(const KArgs &a, const Plan &pl, int sms, cudaStream_t s)
 {
     static size_t conf[64] = {0};
-    auto kernel = daq_phase_kernel<kPhaseTile, kWin>;
+    auto kernel = daq_phase_kernel<kPhaseTile, kWin, kPlain>;
     cudaError_t e = ensure_smem(kernel, pl.smem, conf);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<KArgs *>(&a)};
@@ -1254,7 +1255,7 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     const Plan twopass = pl;
     if (p.grid == 0 && aligned && !skip_isl && !(p.flags & DAQ_SPARSE) && !p.trace && n_fills <= kPlanSmem &&
         (p.wait_limit_ns == 0 || p.wait_limit_ns >= kPhaseMinWaitNs) &&
-        pl.max_tiles >= (int64_t)(pl.halo_free ? kPhaseMinTilesHaloFree : kPhaseMinTiles) * di.sms) {
+        pl.max_tiles >= (int64_t)phase_min_tiles(pl, n_xtal) * di.sms) {
         if (phase_geometry(&pl, p.pre, p.post, n_xtal) && (int)pl.smem <= di.smem_optin) geometry();
         else pl = twopass;
     }
@@ -1336,7 +1337,9 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     const int64_t tiles_cap = std::max<int64_t>(1, std::min<int64_t>(pl.max_tiles, INT32_MAX));
     cudaError_t e = cudaSuccess;
     if (pl.mode == kModePhased) {
-        e = p.pre + p.post <= 32 ? launch_phase<kWin32>(a, pl, di.sms, s) : launch_phase<kWin96>(a, pl, di.sms, s);
+        const bool plain = !pl.need_sarr && !(p.flags & DAQ_DEBUG_CHECKS);
+        if (p.pre + p.post <= 32) e = plain ? launch_phase<kWin32, true>(a, pl, di.sms, s) : launch_phase<kWin32, false>(a, pl, di.sms, s);
+        else e = plain ? launch_phase<kWin96, true>(a, pl, di.sms, s) : launch_phase<kWin96, false>(a, pl, di.sms, s);
         if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
             // fewer SMs for this caller than the device has: the two-pass form runs on any number
             cudaGetLastError();

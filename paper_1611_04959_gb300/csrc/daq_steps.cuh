@@ -477,6 +477,7 @@ __device__ __forceinline__ void sum_pass_step(const KArgs &a, const TileInfo &T,
 // 54 4-byte loads: the count kernel takes 219 us instead of 229 on 24 x 54 x
 // 560,000 samples and 882 instead of 942 on four such fills with the halo-free
 // plan (6.6 TB/s of samples; with its halo the first reads 7.3 TB/s).
+template <bool kPlain = false>
 __device__ __forceinline__ void sum_step_quarters(const KArgs &a, const TileInfo &T, uint32_t slot_s, int it, int nbt,
                                                   uint8_t *abyte, int32_t *blocksum, int32_t *sarr, int lane)
 {
@@ -533,7 +534,7 @@ __device__ __forceinline__ void sum_step_quarters(const KArgs &a, const TileInfo
         abyte[8 * it + g] = (uint8_t)bits;
         if (proper) blocksum[cp >> 3] = sv;
     }
-    if (a.need_sarr && proper) {
+    if (!kPlain && a.need_sarr && proper) {
         if (t < T.t_end) sarr[cp] = S0;
         if (t + 1 < T.t_end) sarr[cp + 1] = S1;
     }
@@ -983,7 +984,7 @@ __device__ __forceinline__ void copy_out(const KArgs &a, const unsigned char *st
 // --------------------------------------------------------------------------- island records (one warp)
 // One record per island end inside the tile.  An island that began in an
 // earlier tile starts at t0 - excl.tr (the marked run entering the tile).
-template <int TW>
+template <int TW, bool kPlain = false>
 __device__ __forceinline__ void write_headers(const KArgs &a, const TileInfo &T, TileWords w, const Agg &excl,
                                               int lane)
 {
@@ -1003,7 +1004,7 @@ __device__ __forceinline__ void write_headers(const KArgs &a, const TileInfo &T,
         const long long t_e = T.t0 + 32 * lane + b;
         const long long ilen = t_e - start + 1;
         const long long row_end = excl.m + w.mb[lane] + __popc(Mt & upto) - 1;
-        if ((a.flags & DAQ_DEBUG_CHECKS) &&
+        if (!kPlain && (a.flags & DAQ_DEBUG_CHECKS) &&
             !(idx >= 0 && T.f >= 0 && T.f < a.n_fills && T.c >= 0 && T.c < a.n_calo && start >= 0 && ilen >= 1 &&
               t_e < T.len && row_end - ilen + 1 >= 0 && row_end - ilen + 1 <= row_end)) {
             set_status_bit(a, DAQ_DEV_BAD_INDEX);  // the record would not describe the fill: skip it
@@ -1024,8 +1025,11 @@ __device__ __forceinline__ void write_headers(const KArgs &a, const TileInfo &T,
 }
 
 // --------------------------------------------------------------------------- Q decimation + fill sum
+// kPlain here and above: a kernel for calls without DAQ_DEBUG_CHECKS whose decimations
+// are all multiples of 8 leaves the other cases' code out.
 // Partial bins of the tile (a group of nthr threads): B_D[k] restricted to the
 // tile, added atomically to the calorimeter's int64 histogram.
+template <bool kPlain = false>
 __device__ __forceinline__ void q_partial(const KArgs &a, const TileInfo &T, const int32_t *blocksum,
                                           const int32_t *sarr, int gt, int nthr)
 {
@@ -1041,12 +1045,12 @@ __device__ __forceinline__ void q_partial(const KArgs &a, const TileInfo &T, con
         for (uint32_t k = k_lo + (uint32_t)gt; k <= k_hi; k += (uint32_t)nthr) {
             const uint32_t lo = max(k * D, t0) - t0, hi = min(k * D + D, t_end) - t0;
             long long sum = 0;
-            if ((D & 7u) == 0u) {
+            if (kPlain || (D & 7u) == 0u) {
                 for (uint32_t b = lo >> 3; b < (hi + 7u) >> 3; ++b) sum += blocksum[b];
             } else {
                 for (uint32_t t = lo; t < hi; ++t) sum += sarr[t];
             }
-            if ((a.flags & DAQ_DEBUG_CHECKS) &&
+            if (!kPlain && (a.flags & DAQ_DEBUG_CHECKS) &&
                 !((long long)k < a.qbins[d] && a.calo_base + T.c >= 0 && a.calo_base + T.c < a.q_calos)) {
                 set_status_bit(a, DAQ_DEV_BAD_INDEX);
                 continue;

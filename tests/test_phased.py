@@ -57,6 +57,10 @@ def run(env, x, lens, grid, rows, hdrs, **kw):
     (2, 4, 54, 140_000, None, dict(NOMINAL, threshold=30_000), 0.0),
     (1, 4, 48, 239_000, None, dict(NOMINAL, decim=(100, 7), ped_samples=1000), 0.03),
     (1, 24, 54, 140_000, None, NOMINAL, 0.0005),
+    (1, 4, 2, 239_000, None, dict(NOMINAL, threshold=100, decim=(8,)), 0.004),
+    (2, 7, 4, 70_000, [70_000, 69_999], NOMINAL, 0.004),
+    (1, 12, 22, 80_648, None, dict(NOMINAL, decim=(100,)), 0.004),
+    (1, 4, 36, 250_000, None, WIDE, 0.001),
 ])
 def test_matches_two_pass(env, F, C, X, N, lens, params, rate):
     torch, daq = env["torch"], env["daq"]
@@ -75,7 +79,7 @@ def test_matches_two_pass(env, F, C, X, N, lens, params, rate):
 @pytest.mark.parametrize("X,params", [(54, WIDE), (40, WIDE), (54, WIDER), (56, WIDER)])
 @pytest.mark.parametrize("N,lens", [(35_000, None), (34_728, [34_728, 11_000]), (35_840, [35_840, 0])])
 def test_wide_windows_match_oracle(env, X, params, N, lens):
-    """post = 64: from 2 tiles an SM on."""
+    """post = 64: from 2 tiles an SM on (48 crystals; 40 stay with the two-pass form)."""
     torch, oracle, daq = env["torch"], env["oracle"], env["daq"]
     x = draw(torch, 2, 2, X, N, seed=X + N, rate=0.002)
     ref = oracle.process_fills(x.cpu().numpy(), params, fill_len=lens, n_threads=8)
