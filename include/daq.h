@@ -121,7 +121,7 @@ typedef struct daq_island {
  *                     form (count kernel, scan, compact kernel), grids from
  *                     occupancy.  The phased form is one cooperative launch
  *                     that compacts each tile a few tiles behind its count, so
- *                     that the second read is from L2: 0.50 ms against 0.66 on
+ *                     that the second read is from L2: 0.49 ms against 0.66 on
  *                     24 x 54 x 560,000 samples.  It takes calls that write
  *                     islands, without DAQ_SPARSE or a trace, of 16-byte
  *                     aligned rows (n_samples % 8 == 0), an even n_xtal of at

@@ -6,7 +6,7 @@
 // pool once (6.5 TB/s over both kernels on a full fill).  Here chunk k is one tile for
 // each CTA, one CTA per SM, and a tile is compacted while at most kPhaseAhead chunks
 // of 152 x 48 KB lie between its two reads.  On 24 x 54 x 560,000 samples HBM reads
-// fall from 2.9 to 1.5 GB (the samples are 1.45) and a fill from 657 to 500 us.
+// fall from 2.9 to 1.5 GB (the samples are 1.45) and a fill from 657 to 487 us.
 //
 // Warps of a CTA, handing tiles on through mbarriers:
 //   8 sum        crystal sums, threshold bits and block sums of a tile in one of two
@@ -35,7 +35,8 @@
 // for odd crystal counts took a fill from 652 to 552 us, Q bins in 32-bit arithmetic
 // and a kernel for each kind of window (kWin32, kWin96: one form of marks_word each)
 // from there to 516, kernels without the code for DAQ_DEBUG_CHECKS and odd decimations
-// (kPlain) to 500.  At 552: counting by 4 warps 565; kPhaseAhead 4: 754, 5 to 7: 552.
+// (kPlain) to 500.  With that, kPhaseAhead 6 instead of 5 takes it to 487 (7: 503; little
+// noise 333 against 373, post = 64 504 against 565).  At 552: counting by 4 warps 565; kPhaseAhead 4: 754, 5 to 7: 552.
 // The two jobs in turn by the same warps, two CTAs per SM: 635 at best.
 #pragma once
 
@@ -44,7 +45,7 @@
 namespace daq {
 
 constexpr int kPhaseTile = 448;    // samples per tile
-constexpr int kPhaseAhead = 5;     // tiles of a CTA between a tile's count and the end of its compaction
+constexpr int kPhaseAhead = 6;     // tiles of a CTA between a tile's count and the end of its compaction
 constexpr unsigned kPhasePoll = 100;  // ns between reads of a chunk's words
 constexpr int kPhaseInfo = kPhaseAhead + 1;     // tile records: one more is decoded ahead
 constexpr int kPhaseXtal = 56;             // crystals it takes (a multiple of 4): four slots fit up to here
