@@ -45,8 +45,9 @@ def measured_peaks() -> tuple:
         return 6800.0, "fallback"
 
 
-# Sources compiled into the two-pass kernels (prepare, count, scan, compact).
-KERNEL_SOURCES = ("daq_device.cuh", "daq_steps.cuh", "daq_twopass.cuh", "daq_process.cu")
+# Sources compiled into the default forms' kernels (prepare, phased; count, scan, compact).
+KERNEL_SOURCES = ("daq_device.cuh", "daq_steps.cuh", "daq_twopass.cuh", "daq_phase.cuh", "daq_launch.cuh",
+                  "daq_process.cu")
 
 
 def kernel_source_hash() -> str:
@@ -262,7 +263,8 @@ def bench_gb300(args, ws, rank, local):
     elapsed_ms = t_start.elapsed_time(t_end)
 
     # ---- per-kernel times and per-step latency: a second run with DAQ_N_EVENTS events per step
-    # [0] start, [1] after pedestals, [2] after count kernel, [3] after scan, [4] end
+    # [0] start, [1] after pedestals, [2] after count kernel, [3] after scan, [4] end (the
+    # phased form's one kernel: [2] to [4] after it)
     # (the events cost about 10 us per step, so they stay out of the timed region)
     Kd = max(3, min(K, 500))
     NE = 5
@@ -277,22 +279,21 @@ def bench_gb300(args, ws, rank, local):
             call(p, ctypes.cast(ev_arrays[k], ctypes.c_void_p).value)
     torch.cuda.synchronize(dev)
     step_ms = [e[0].elapsed_time(e[4]) for e in evs]
-    prep_ms = [e[0].elapsed_time(e[1]) for e in evs]
-    count_ms = [e[1].elapsed_time(e[2]) for e in evs]
-    scan_ms = [e[2].elapsed_time(e[3]) for e in evs]
-    compact_ms = [e[3].elapsed_time(e[4]) for e in evs]
+    kern = kernel_means(evs)
     _, elapsed_ms, value = replicas.aggregate(K * raw_bytes, elapsed_ms, dev)
 
-    # ---- roofline of the dominant kernel: the compact pass (reads the samples, writes the islands)
+    # ---- roofline of the dominant kernel: the phased kernel (reads the samples once from HBM, adds to Q,
+    # writes the islands) or the compact pass (reads the samples, writes the islands)
     peak, peak_kind = measured_peaks()
     q_bytes = sum(C * daq.daq_q_bins(N, d) * 16 for d in params["decim"])
     n_tiles = F * C * (-(-N // 448))
     side = n_tiles * (14 * 4 + 16 + 16)             # marks words, aggregate, prefix per tile
-    alg_count = raw_bytes + q_bytes + side
-    alg_compact = raw_bytes + n_rows * X * 2 + n_isl * 24 + side
-    count_mean, compact_mean = statistics.fmean(count_ms), statistics.fmean(compact_ms)
-    achieved = alg_compact / (compact_mean * 1e-3) / 1e9
-    traffic = profiled_traffic("daq_compact_kernel", "full_fill")
+    islands_bytes = n_rows * X * 2 + n_isl * 24
+    phased = "daq_phase_kernel" in kern
+    top = "daq_phase_kernel" if phased else "daq_compact_kernel"
+    alg = raw_bytes + islands_bytes + (q_bytes + 4 * n_tiles if phased else side)
+    achieved = alg / (kern[top] * 1e-3) / 1e9
+    traffic = profiled_traffic(top, "full_fill")
 
     result = {
         "metric": METRIC, "value": round(value, 2), "unit": UNIT, "n_gpus": ws, "steps": K,
@@ -302,24 +303,21 @@ def bench_gb300(args, ws, rank, local):
                                f"({raw_bytes / 1e9:.4f} GB), literal noise sigma 3/crystal, T=30, pre=8, post=24, D=32",
                    "fills_per_step_per_gpu": 1, "raw_bytes_per_step_per_gpu": raw_bytes,
                    "l2": "inputs larger than L2 (1.45 GB per step vs 129 MB)", "parallelism": f"replicas x{ws}",
-                   "tile": 448, "form": "two-pass: count kernel, scan, compact kernel"},
+                   "tile": 448, "form": "phased: count and compaction in one kernel, second read from L2" if phased
+                   else "two-pass: count kernel, scan, compact kernel"},
         "pct_of_hbm_peak": round(100.0 * value / ws / peak, 2),
         "pct_of_nominal_hbm": round(100.0 * value / ws / NOMINAL_HBM_GBS, 2),
         "latency_ms": {"p50": round(statistics.median(step_ms), 4),
                        "p99": round(float(np.percentile(step_ms, 99)), 4),
                        "max": round(max(step_ms), 4)},
-        "kernels_ms": {"daq_prepare_kernel": round(statistics.fmean(prep_ms), 4),
-                       "daq_count_kernel": round(count_mean, 4),
-                       "daq_scan_kernel": round(statistics.fmean(scan_ms), 4),
-                       "daq_compact_kernel": round(compact_mean, 4)},
-        "count_kernel_gbs": round(alg_count / (count_mean * 1e-3) / 1e9, 1),
+        "kernels_ms": kern,
         "islands_per_fill": n_isl, "pool_rows_per_fill": n_rows,
         "coverage": round(n_rows / (C * N), 4),
         "output_over_input": round((n_rows * X * 2 + n_isl * 24) / raw_bytes, 4),
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": traffic, "peak_source": peak_kind,
-                     "kernel": "daq_compact_kernel", "algorithmic_bytes_per_launch": alg_compact},
-        "gpu_launches": 4 * K,
+                     "kernel": top, "algorithmic_bytes_per_launch": alg},
+        "gpu_launches": len(kern) * K,
         "clocks": clocks.summary(),
     }
 
@@ -547,9 +545,11 @@ def bench_batched(args, torch, dev, daq, synth, W, w=None, plain_flags=0) -> dic
     plain_ms = p0.elapsed_time(p1)
     plain = {"value": round(Kb * raw / (plain_ms * 1e-3) / 1e9, 2), "unit": UNIT, "steps": Kb,
              "ms_per_batch": round(plain_ms / Kb, 4),
-             "form": "default two-pass kernels, one daq_process_fills call per fill (16 calls per batch), "
+             "form": "default kernels, one daq_process_fills call per fill (16 calls per batch), "
                      "no graph, no tuning" + (f", flags {plain_flags}" if plain_flags else "")}
     del ws1
+    # prepare and phased kernel, or prepare, count, scan and compact
+    per_batch = 2 if tuning["grid"] == 0 and tuning["tile"] in (0, 448) and not tuning.get("flags", 0) & daq.DAQ_SPARSE else 4
     res = {"value": round(Kb * raw / (total_ms * 1e-3) / 1e9, 2), "unit": UNIT, "steps": Kb,
            "ms_per_batch": round(total_ms / Kb, 4),
            "latency_ms": {"p50": round(statistics.median(ms), 4), "p99": round(float(np.percentile(ms, 99)), 4)},
@@ -564,7 +564,7 @@ def bench_batched(args, torch, dev, daq, synth, W, w=None, plain_flags=0) -> dic
                      "candidates": tuning["n_tried"],
                      "ms": round(tuning["ms"], 4), "ms_default_config": round(tuning["ms_default"], 4),
                      "tuning_s": round(tune_s, 2)},
-           "gpu_launches": 4 * Kb, "generation_s": round(gen_s, 1),
+           "gpu_launches": per_batch * Kb, "generation_s": round(gen_s, 1),
            "plain_form": plain, "batched_over_plain": round((Kb * raw / (total_ms * 1e-3)) / (Kb * raw / (plain_ms * 1e-3)), 4)}
     del samples, out, q
     torch.cuda.empty_cache()
@@ -618,6 +618,17 @@ def copy_bandwidth(torch, dev, host_in, dev_in, host_out, dev_out, out_rows: int
                       "(d2h), alone and concurrently on two streams"}
 
 
+def kernel_means(evs) -> dict:
+    """Mean ms of each kernel of a call from its DAQ_N_EVENTS events per step.  The
+    phased form records the last three after its one kernel, so nothing lies
+    between them (a compact kernel takes longer than a few microseconds)."""
+    mean = [statistics.fmean(r[i].elapsed_time(r[i + 1]) for r in evs) for i in range(4)]
+    names = ["daq_prepare_kernel", "daq_count_kernel", "daq_scan_kernel", "daq_compact_kernel"]
+    if mean[3] < 0.004:
+        names = ["daq_prepare_kernel", "daq_phase_kernel"]
+    return {name: round(ms, 4) for name, ms in zip(names, mean)}
+
+
 def time_calls(torch, dev, daq, x, F, C, X, N, params, K: int, out=None, warm: int = 2):
     """Run daq_process_fills K times on device samples x[F][C][X][N].  Returns
     (total ms of the K calls, per-step ms list and kernel means from a second
@@ -657,9 +668,7 @@ def time_calls(torch, dev, daq, x, F, C, X, N, params, K: int, out=None, warm: i
     p.events = None
     torch.cuda.synchronize(dev)
     ms = [r[0].elapsed_time(r[4]) for r in evs]
-    kern = {name: round(statistics.fmean(r[i].elapsed_time(r[i + 1]) for r in evs), 4)
-            for i, name in enumerate(["daq_prepare_kernel", "daq_count_kernel", "daq_scan_kernel",
-                                      "daq_compact_kernel"])}
+    kern = kernel_means(evs)
     counts = out.counts.cpu().numpy()
     del ws, q
     return total, ms, kern, counts
@@ -700,7 +709,7 @@ def bench_sparse(args, torch, dev, daq, synth, W) -> dict:
             "pct_of_hbm_peak": round(100.0 * value / peak, 2),
             "two_pass_ceiling_gbs": round(ceiling, 1), "frac_of_two_pass_ceiling": round(value / ceiling, 4),
             "read_once_ceiling_gbs": round(once, 1), "frac_of_read_once_ceiling": round(value / once, 4),
-            "kernels_ms": kern, "gpu_launches": 4 * K,
+            "kernels_ms": kern, "gpu_launches": len(kern) * K,
             "default_flags": {"value": round(K * raw / (total_d * 1e-3) / 1e9, 2), "ms_per_step": round(total_d / K, 4),
                               "kernels_ms": kern_d}}
 
@@ -752,7 +761,7 @@ def bench_stress(args, torch, dev, daq, synth, W) -> dict:
                        "fills cycle over 4 distinct generated fills",
            "raw_bytes_per_batch": raw, "islands_per_batch": int(counts[0]), "pool_rows_per_batch": int(counts[1]),
            "coverage": round(int(counts[1]) / (F * C * N), 6), "status": status,
-           "output_sizes": "computed on the device (counts) in the same call", "gpu_launches": 4 * Ks,
+           "output_sizes": "computed on the device (counts) in the same call", "gpu_launches": len(kern) * Ks,
            "kernels_ms": kern, "tile": plan_tile(daq, F, C, X, N, params),
            "generation_s": round(gen_s, 1)}
     del x, out
@@ -823,7 +832,7 @@ def bench_pack(args, torch, dev, daq, pool, rows: int) -> dict:
     ms = e0.elapsed_time(e1) / K
     n = int(nbytes.item())
     raw = rows * X * 2
-    alg = 2 * raw + n        # the pool is read by the size pass and by the write pass
+    alg = raw + n            # the pool is read once, the stream written
     peak = measured_peaks()[0]
     # decoding the stream back into pool rows (checked against the pool once)
     back = torch.empty((rows, X), dtype=torch.int16, device=dev)
@@ -852,7 +861,7 @@ def bench_pack(args, torch, dev, daq, pool, rows: int) -> dict:
                          "frac": round(alg / (ms * 1e-3) / 1e9 / peak, 4), "algorithmic_bytes_per_launch": alg},
             "unpack": {"value": round(raw / (ums * 1e-3) / 1e9, 2), "unit": "GB/s of pool rows decoded",
                        "ms_per_fill": round(ums, 4), "steps": K, "gpu_launches": K},
-            "gpu_launches": 5 * K}
+            "gpu_launches": K}
 
 
 THRESHOLDS = (5, 10, 15, 20, 30, 50, 100, 300, 1000)

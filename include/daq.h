@@ -107,8 +107,11 @@ typedef struct daq_island {
  *                count records of the 32 tiles after it at once.  Outputs are
  *                identical with and without it.  Where few tiles hold islands
  *                it halves the compact pass (0.217 -> 0.117 ms on a fill with
- *                8.6% of samples in islands); where nearly all do, the extra
- *                steps cost about 0.5%.  The batch tuner tries both.
+ *                8.6% of samples in islands).  Calls with it take the two-pass
+ *                form: on that fill 0.354 ms against 0.337 for the phased form
+ *                without the flag; at a fifth of its pulses 0.313 against 0.326,
+ *                and several such calls at once overlap better.  The batch
+ *                tuner tries both.
  *   tile         samples per tile: 0 = chosen by the library (two-pass form: the
  *                width of least estimated count-pass cost, 448 for the nominal
  *                windows and 384 when the halo of post + pre samples is too
@@ -259,7 +262,8 @@ int64_t daq_q_bins(int64_t n_samples, int32_t decim);
  *   samples      device int16[n_fills][n_calo][n_xtal][n_samples] (row pitch
  *                n_samples; 12-bit ADC values in 16-bit words, Sec. 3); the
  *                fast path wants 16-byte aligned rows (n_samples % 8 == 0);
- *                other pitches cost the two-pass form about 1.7x a sample.
+ *                other pitches cost the two-pass form more a sample (191 us
+ *                on 24 x 54 x 100,003).
  *   n_xtal       crystals per calorimeter, 1..64 (the experiment has 54, Sec. 3).
  *   qhist_inout  device int64 Q histograms (layout: see daq_q_bins); B_D[k] =
  *                sum of S over samples [kD, min(kD + D, len)) is ADDED to bin k

@@ -6,7 +6,7 @@
 // pool once (6.5 TB/s over both kernels on a full fill).  Here chunk k is one tile for
 // each CTA, one CTA per SM, and a tile is compacted while at most kPhaseAhead chunks
 // of 152 x 48 KB lie between its two reads.  On 24 x 54 x 560,000 samples HBM reads
-// fall from 2.9 to 1.5 GB (the samples are 1.45) and a fill from 657 to 487 us.
+// fall from 2.9 to 1.6 GB (the samples are 1.45) and a fill from 657 to 487 us.
 //
 // Warps of a CTA, handing tiles on through mbarriers:
 //   8 sum        crystal sums, threshold bits and block sums of a tile in one of two
@@ -35,9 +35,9 @@
 // for odd crystal counts took a fill from 652 to 552 us, Q bins in 32-bit arithmetic
 // and a kernel for each kind of window (kWin32, kWin96: one form of marks_word each)
 // from there to 516, kernels without the code for DAQ_DEBUG_CHECKS and odd decimations
-// (kPlain) to 500.  With that, kPhaseAhead 6 instead of 5 takes it to 487 (7: 503; little
-// noise 333 against 373, post = 64 504 against 565).  At 552: counting by 4 warps 565; kPhaseAhead 4: 754, 5 to 7: 552.
-// The two jobs in turn by the same warps, two CTAs per SM: 635 at best.
+// (kPlain) to 500.  With that, kPhaseAhead 6 instead of 5 takes it to 487 (4: 709, 7: 503;
+// little noise 333 against 373, post = 64 504 against 565).  At 552, counting by 4 warps
+// took 565.  The two jobs in turn by the same warps, two CTAs per SM: 635 at best.
 #pragma once
 
 #include "daq_twopass.cuh"

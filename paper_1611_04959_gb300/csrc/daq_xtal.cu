@@ -6,9 +6,9 @@
 // with P the per-crystal pedestal of Table 2's pedestal kernel (the first
 // min(ped_samples, len) samples, rounded half up).  Q stays on the device and
 // accumulates over calls.  Two kernels: pedestals (one warp per crystal row),
-// then a streaming pass in which each thread owns 8 consecutive samples of one
-// crystal row, adds every fill of the call in registers and read-modify-writes
-// its 8 int64 accumulators once.  HBM traffic per call: the samples once
+// then a streaming pass in which each thread owns groups of 8 consecutive samples
+// of the rows taken as one flat sequence, adds every fill of the call in registers
+// and read-modify-writes the 8 int64 accumulators once.  HBM traffic per call: the samples once
 // (2 bytes each) and Q once each way (16 bytes per crystal-sample).
 #include <cuda_runtime.h>
 
