@@ -401,7 +401,7 @@ int daq_process_fills_static(const int16_t *samples, int n_calo, int n_xtal, int
  *                plan then allocates and owns one.  With DAQ_TUNE, params->tile
  *                and params->grid are ignored and chosen by the tuner, and so
  *                is the DAQ_SPARSE bit of params->flags.
- *   plan_flags   DAQ_TUNE: time the candidate configurations (two-pass form at
+ *   plan_flags   DAQ_TUNE: time the candidate configurations (default form at
  *                the library's tile, with and without DAQ_SPARSE, and at tile
  *                widths 128/224/384/448 with 2 or 1 CTAs per SM; the
  *                single-launch form at 448) on this batch and keep the

@@ -53,7 +53,7 @@ struct Candidate {
     uint32_t flags;  // DAQ_SPARSE or 0
 };
 
-// Form x tile x CTAs: the default (two-pass, tile chosen by the library), the
+// Form x tile x CTAs: the default (phased or two-pass, tile chosen by the library), the
 // same with the compact pass that passes over tiles without marks (DAQ_SPARSE),
 // the two-pass form at 128 / 224 / 384 / 448 with occupancy grids (2 CTAs per
 // SM) and with one CTA per SM, and the single-launch form at 448.  The single-pass

@@ -1,5 +1,5 @@
-// Two-pass form of the per-fill processing (the default path), and its
-// single-launch variant.
+// Two-pass form of the per-fill processing (the default where the phased form, see
+// daq_phase.cuh, does not apply or pay), and its single-launch variant.
 //
 //   daq_count_kernel    every tile once, with its halo: crystal sums, pedestal
 //                       subtraction, threshold, pre/post windows (the marks of
