@@ -893,6 +893,16 @@ int pipelined_grid(int slot, K kernel, int X, int threads, size_t smem, size_t s
     return (int)std::max<long long>(1, std::min<long long>(want, (long long)resident));
 }
 
+// The most shared memory a warp of a kernel takes, over the crystal counts.  Not the
+// plan of the most crystals: 64 columns side by side are also 16 blocks of 4 crystals,
+// and an encoder stage keeps a word for each block.
+template <typename F> size_t most_bytes(F bytes_of)
+{
+    size_t most = 0;
+    for (int X = 1; X <= kMaxX; ++X) most = std::max(most, bytes_of(X));
+    return most;
+}
+
 // Workspace: one status word per chunk, then the ticket and the role counter.
 long long enc_chunks(long long nb, int X) { return (nb + EncPlan(X).chunk_blocks() - 1) / EncPlan(X).chunk_blocks(); }
 size_t pack_ws(long long nb, int X) { return (8 * (size_t)(enc_chunks(nb, X) + 2) + 255) & ~size_t(255); }
@@ -931,7 +941,8 @@ int daq_pack_pool(const int16_t *pool, int64_t rows, int n_xtal, void *out, int6
     const long long n_chunks = enc_chunks(nb, n_xtal);
     const bool even = (n_xtal % 2) == 0;
     const auto kernel = even ? pack_kernel<true> : pack_kernel<false>;
-    const size_t smem = kEncWarps * EncPlan(n_xtal).bytes(), most = kEncWarps * EncPlan(kMaxX).bytes();
+    static const size_t warp_most = most_bytes([](int X) { return EncPlan(X).bytes(); });
+    const size_t smem = kEncWarps * EncPlan(n_xtal).bytes(), most = kEncWarps * warp_most;
     const int grid = pipelined_grid(even ? 0 : 1, kernel, n_xtal, kEncThreads, smem, most, n_chunks + 1);
     if (grid < 1) return DAQ_ECUDA;
     if (cudaMemsetAsync(workspace, 0, 8 * (size_t)(n_chunks + 2), s) != cudaSuccess) return DAQ_ECUDA;
@@ -953,7 +964,8 @@ int daq_unpack_pool(const void *in, int64_t in_bytes, int64_t rows, int n_xtal, 
     const bool even = (n_xtal % 2) == 0;
     const auto kernel = even ? unpack_kernel<true> : unpack_kernel<false>;
     const DecPlan pl(n_xtal);
-    const size_t most = kDecWarps * DecPlan(kMaxX).bytes(kMaxX);
+    static const size_t warp_most = most_bytes([](int X) { return DecPlan(X).bytes(X); });
+    const size_t most = kDecWarps * warp_most;
     const int grid = pipelined_grid(even ? 2 : 3, kernel, n_xtal, kDecThreads, kDecWarps * pl.bytes(n_xtal), most,
                                     (std::max<long long>(nb, 1) + kDecWarps * pl.G - 1) / (kDecWarps * pl.G));
     if (grid < 1) return DAQ_ECUDA;
