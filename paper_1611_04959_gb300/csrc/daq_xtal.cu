@@ -119,12 +119,14 @@ __device__ __forceinline__ void store_q(long long *p, const long long (&v)[8], b
 // rate) against 2.17 with accesses of 16 bytes, 64 apart from lane to lane, and
 // 3.03 with lanes on consecutive 16 bytes and 4-byte sample loads.  Groups within a
 // row, taken sample by sample where the pitch is odd, took 1.70 ms for three fills of
-// 24 x 54 x 99,999; these take 0.48.  Four CTAs an SM: at five the 64 registers do
+// 24 x 54 x 99,999; these take 0.45.  A sample past its fill's length is not read:
+// eight fills of 24 x 54 x 70,000 cut to 7,000 take 262 us, 465 if it is.  Four CTAs an SM: at five the 64 registers do
 // not suffice (2.22 ms).
 // kVec: aligned 16-byte sample loads, of kAhead fills at once (two: 721 us for four
 // fills of 140,000 samples against 731 with one and 748 with four, whose registers
-// cost a CTA); wide: q is 32-byte aligned.  I: the index type, 32 bits where the
-// cells allow (one division a group).
+// cost a CTA); wide: q is 32-byte aligned.  I: the type of rows and places in them, 32
+// bits where the cells allow (one division a group, and the compares with every
+// fill's length: those four fills take 674 us so).
 template <bool kVec, int kAhead, typename I>
 __global__ void __launch_bounds__(kThreads, 4) xtal_sum_kernel(const int16_t *samples, int n_fills, int n_calo,
                                                             int n_xtal, int64_t pitch, const int32_t *lens,
@@ -136,9 +138,9 @@ __global__ void __launch_bounds__(kThreads, 4) xtal_sum_kernel(const int16_t *sa
     for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < groups; i += (long long)gridDim.x * kThreads) {
         const long long at = 8 * i;
         const I row = (I)at / (I)pitch;
-        const long long t0 = at - (long long)row * pitch;
+        const I t0 = (I)at - row * (I)pitch;
         const bool full = at + 8 <= cells;
-        const bool one_row = full && t0 + 8 <= pitch;
+        const bool one_row = full && (long long)t0 + 8 <= pitch;
         long long acc[8];
         if (full) {  // the accumulators' loads go out before the samples'
             load_q(q + at, acc, wide);
@@ -148,17 +150,17 @@ __global__ void __launch_bounds__(kThreads, 4) xtal_sum_kernel(const int16_t *sa
         }
         for (int f0 = 0; f0 < n_fills; f0 += kAhead) {
             int4 v[kAhead];
-            if (kVec && full) {
+            if (kVec && one_row) {
 #pragma unroll
                 for (int u = 0; u < kAhead; ++u)
-                    if (f0 + u < n_fills)
+                    if (f0 + u < n_fills && t0 + 8 <= (I)lens[f0 + u])
                         v[u] = __ldcs(reinterpret_cast<const int4 *>(samples + (long long)(f0 + u) * cells + at));  // read once
             }
 #pragma unroll
             for (int u = 0; u < kAhead; ++u) {
                 const int f = f0 + u;
                 if (f >= n_fills) break;
-                const long long len = lens[f];
+                const I len = (I)lens[f];
                 const int32_t *P = ped + (long long)f * n_rows + row;
                 if (kVec && one_row && t0 + 8 <= len) {
                     const int p = P[0];
@@ -171,12 +173,12 @@ __global__ void __launch_bounds__(kThreads, 4) xtal_sum_kernel(const int16_t *sa
                 } else if (!one_row || t0 < len) {
                     // the end of a row, of the fill or of the array
                     const int16_t *src = samples + (long long)f * cells + at;
-                    long long t = t0;
+                    I t = t0;
                     int r = 0;
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         if (at + k < cells && t < len) acc[k] += (int)src[k] - P[r];
-                        if (++t == pitch) {
+                        if (++t == (I)pitch) {
                             t = 0;
                             ++r;
                         }
