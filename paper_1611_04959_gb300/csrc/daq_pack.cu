@@ -110,27 +110,43 @@ __device__ __forceinline__ void swap_bits8(uint32_t (&p)[8])
 // the sign plane xor the others gives the zigzag planes, whose highest non-zero
 // one is the width.  Where a column of the round is wider (pulses: 3% of the
 // blocks of a dense fill, most of those early in a fill), all take 16-bit
-// differences and the swaps on low and high bytes; differences past 16 bits are
-// done a column at a time by the whole warp.  (Every chunk waits for the slowest
-// before it, so a slow round costs more than its share: with one column at a
+// differences and the swaps on low and high bytes, with the differences' signs,
+// which 16 bits may not hold, as a plane of their own.  (Every chunk waits for the
+// slowest before it, so a slow round costs more than its share: with one column at a
 // time for all wide ones the pass took 543 us, with every column of such a round
 // sample by sample 646.)  The words' places within the block are
 // one scan over the lanes.
+//
+// A round of noise takes some 6 words a column, one of wide columns up to 18.  The
+// staged words of a warp are a ring that holds six of the first or two of the last: a
+// round begins at the next free unit, and the oldest rounds are written out early where
+// there is no piece for what the last round took.  2 M rows x 54, us for noise of
+// sigma 3 / 8 / 24 and for full-range samples: 90 / 91 / 152 / 169.  (Six stages of
+// seven words a column, rounds that did not fit encoded a second time from rows read
+// again, and one column at a time for differences past 16 bits: 90 / 164 / 295 / 1707;
+// the three kernels before: 164 / 164 / 217 / 243.  Emptying the ring and changing the
+// stages' size: 350 at sigma 7, where every other round needs it.)
 constexpr int kEncWarps = 8;
 constexpr int kEncThreads = 32 * kEncWarps;
-constexpr int kEncDepth = 6;  // stages of a warp
+constexpr int kEncDepth = 6;  // rounds of a warp that are encoded or written out
+constexpr int kEncWarpBytes = 14336;  // shared memory of a warp with which two CTAs share an SM
+constexpr int kEncUnits = 12;  // units of the ring of staged words
 constexpr int kEncRing = 16;  // chunks whose tickets and sizes a CTA remembers: at least 2 kEncDepth + 3
 
-// Shared memory of one encoder warp: its stages, what they hold, a round's rows
-// and their barrier.
+// Shared memory of one encoder warp: a ring of encoded words, a round's rows, where in
+// the ring the rounds lie, and the rows' barrier.
 struct EncPlan : Lanes {
-    int cap, inb;  // bytes of a stage, of a round's rows
+    int unit, inb;  // words of a unit of the ring, bytes of a round's rows
+    // Units of four words a column (two hold a column of 7 planes, five any), or of as
+    // many from three and a half on as let two CTAs share an SM; where none do, four again.
     __host__ __device__ explicit EncPlan(int X) : Lanes(X)
     {
-        cap = (28 * nsub * X + 15) & ~15;  // seven words a column; rounds that do not fit are encoded again into place
-        inb = nsub * 64 * X;
+        const int cols = nsub * X, least = (7 * cols + 1) / 2;
+        inb = 64 * cols;
+        const int fit = (kEncWarpBytes - inb - 4 * kEncDepth * (1 + nsub) - 48) / (4 * kEncUnits);
+        unit = fit < least || fit > 4 * cols ? 4 * cols : fit;
     }
-    __host__ __device__ size_t rows_at() const { return (size_t)kEncDepth * cap; }
+    __host__ __device__ size_t rows_at() const { return (4 * (size_t)kEncUnits * unit + 15) & ~size_t(15); }
     __host__ __device__ size_t meta_at() const { return rows_at() + (size_t)inb; }
     __host__ __device__ size_t bar_at() const { return meta_at() + 4 * (size_t)kEncDepth * (1 + nsub); }
     __host__ __device__ size_t bytes() const { return ((bar_at() + 15) & ~size_t(15)) + 16; }
@@ -224,14 +240,6 @@ __device__ long long enc_places(unsigned long long *st, long long n_chunks)
     return at;
 }
 
-// Zigzag code of this lane's row of a column (pitch X; the warp, lanes on rows).
-__device__ __forceinline__ uint32_t row_code(const int16_t *col, int X, int lane)
-{
-    const int32_t v = col[lane * X];
-    const int32_t prev = __shfl_up_sync(kFull, v, 1);
-    return lane ? zigzag(v - prev) : 0u;
-}
-
 // a - b in every byte, modulo 256.
 __device__ __forceinline__ uint32_t sub8x4(uint32_t a, uint32_t b)
 {
@@ -263,25 +271,27 @@ __device__ __forceinline__ uint32_t sub16x2(uint32_t v, uint32_t p)
     return ((v | 0x80008000u) - (p & 0x7fff7fffu)) ^ ((v ^ ~p) & 0x80008000u);
 }
 
-// The zigzag planes 0..15 (lo, hi) of one column from the low and high bytes of
-// its differences, in place; returns the width.  All differences fit 16 bits.
-__device__ __forceinline__ int word_planes(uint32_t (&lo)[8], uint32_t (&hi)[8])
+// The zigzag planes of one column from the low and high bytes of its differences
+// modulo 2^16 and their signs: planes 0..7 in lo, 8..15 in hi, 16 in sign; returns the
+// width.
+__device__ __forceinline__ int word_planes(uint32_t (&lo)[8], uint32_t (&hi)[8], uint32_t &sign)
 {
     swap_bits8(lo);
     swap_bits8(hi);
-    const uint32_t sign = hi[7];
+    const uint32_t s = sign;
+    sign ^= hi[7];
 #pragma unroll
-    for (int k = 7; k > 0; --k) hi[k] = hi[k - 1] ^ sign;
-    hi[0] = lo[7] ^ sign;
+    for (int k = 7; k > 0; --k) hi[k] = hi[k - 1] ^ s;
+    hi[0] = lo[7] ^ s;
 #pragma unroll
-    for (int k = 7; k > 0; --k) lo[k] = lo[k - 1] ^ sign;
-    lo[0] = sign;
+    for (int k = 7; k > 0; --k) lo[k] = lo[k - 1] ^ s;
+    lo[0] = s;
     int w = 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) w = lo[k] ? k + 1 : w;
 #pragma unroll
     for (int k = 0; k < 8; ++k) w = hi[k] ? k + 9 : w;
-    return w;
+    return sign ? 17 : w;
 }
 
 // Encode `blocks` <= nsub blocks side by side from the rows at `in` (block pitch
@@ -318,102 +328,81 @@ template <bool kEven> struct Round {
     }
 };
 
-// The head word and planes 0 .. 7 of a column at word o; words at or past `room`
-// are dropped.
-__device__ __forceinline__ void store_column(uint32_t *dst, int o, int room, uint32_t first, int w, const uint32_t (&p)[8])
+// The head word and planes 0 .. 7 of a column.
+__device__ __forceinline__ void store_column(uint32_t *dst, uint32_t first, int w, const uint32_t (&p)[8])
 {
-    if (o < room) dst[o] = first | ((uint32_t)w << 16);
-    const int n = min(w, room - o - 1);
+    dst[0] = first | ((uint32_t)w << 16);
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-        if (k < n) dst[o + 1 + k] = p[k];
+        if (k < w) dst[1 + k] = p[k];
 }
 
 // A round with a column that is not narrow.  A function of its own: with both
 // forms in one body the narrow one ran 2.3x slower.  Returns the words of the
-// round and those ahead of the lane's block.
+// round, kWideRound if a column has more than 8 planes, and the words ahead of the
+// lane's block.
+constexpr int kWideRound = 1 << 30;
 template <bool kEven>
-__device__ __noinline__ int2 encode_wide_round(int X, const int16_t *in, int blocks, uint32_t *dst, int fit, int room)
+__device__ __noinline__ int2 encode_wide_round(int X, const int16_t *in, int blocks, uint32_t *dst, int fit)
 {
     const int lane = threadIdx.x & 31;
     const EncPlan pl(X);
     const Round<kEven> R(pl, X, in, blocks, lane);
-    uint32_t p0[8], p1[8], h0[8], h1[8], mx = R.row(0), mn = mx;
+    uint32_t p0[8], p1[8], h0[8], h1[8], s0 = 0, s1 = 0, prev[4];
+    const uint32_t v0 = R.row(0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) prev[j] = j ? R.row(8 * j - 1) : v0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        uint32_t d[4];  // differences of rows k, k + 8, ..., both columns
+        uint32_t d[4], sg[4];  // rows k, k + 8, ..., both columns: differences modulo 2^16, their signs (bits 15 and 31)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const uint32_t v = R.row(8 * j + k);
-            d[j] = 8 * j + k ? sub16x2(v, R.row(8 * j + k - 1)) : 0u;
-            mx = __vmaxs2(mx, v);
-            mn = __vmins2(mn, v);
+            d[j] = sub16x2(v, prev[j]);
+            sg[j] = d[j] ^ ((v ^ prev[j]) & (v ^ d[j]));
+            prev[j] = v;
         }
         const uint32_t t = __byte_perm(d[0], d[1], 0x6240), u = __byte_perm(d[2], d[3], 0x6240);
         const uint32_t th = __byte_perm(d[0], d[1], 0x7351), uh = __byte_perm(d[2], d[3], 0x7351);
+        const uint32_t ts = __byte_perm(sg[0], sg[1], 0x7351), us = __byte_perm(sg[2], sg[3], 0x7351);
         p0[k] = __byte_perm(t, u, 0x5410);
         p1[k] = __byte_perm(t, u, 0x7632);
         h0[k] = __byte_perm(th, uh, 0x5410);
         h1[k] = __byte_perm(th, uh, 0x7632);
+        s0 |= (__byte_perm(ts, us, 0x5410) >> (7 - k)) & (0x01010101u << k);
+        s1 |= (__byte_perm(ts, us, 0x7632) >> (7 - k)) & (0x01010101u << k);
     }
-    int w0 = word_planes(p0, h0), w1 = word_planes(p1, h1);
-    // columns with differences past 16 bits, one at a time by the whole warp
-    const bool past0 = R.mine && (int)(int16_t)(mx & 0xffffu) - (int)(int16_t)(mn & 0xffffu) > 32767;
-    const bool past1 = R.two && ((int)mx >> 16) - ((int)mn >> 16) > 32767;
-    const unsigned m0 = __ballot_sync(kFull, past0), m1 = __ballot_sync(kFull, past1);
-    const int at = (int)(R.col - in);
-    auto widths = [&](unsigned m, int second, int &w) {
-        for (; m; m &= m - 1u) {
-            const int owner = __ffs(m) - 1;
-            const int v = 32 - __clz(__reduce_or_sync(kFull, row_code(in + __shfl_sync(kFull, at, owner) + second, X, lane)));
-            if (lane == owner) w = v;
-        }
-    };
-    widths(m0, 0, w0);
-    widths(m1, 1, w1);
+    const int w0 = word_planes(p0, h0, s0), w1 = word_planes(p1, h1, s1);
     int total, before;
-    const int o0 = R.place(pl, w0, w1, lane, total, before), o1 = o0 + 1 + w0;
-    if (total > fit) return make_int2(total, before);
-    const uint32_t v0 = R.row(0);
-    auto upper = [&](int o, int w, const uint32_t (&h)[8]) {  // planes 8 .. 15
+    const int o0 = R.place(pl, w0, w1, lane, total, before);
+    const int ret = total | (__any_sync(kFull, R.mine && max(w0, w1) > 8) ? kWideRound : 0);
+    if (total > fit) return make_int2(ret, before);
+    auto store = [&](uint32_t *at, uint32_t first, int w, const uint32_t (&p)[8], const uint32_t (&h)[8], uint32_t top) {
+        store_column(at, first, w, p);
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-            if (k + 8 < min(w, room - o - 1)) dst[o + 9 + k] = h[k];
+            if (8 + k < w) at[9 + k] = h[k];
+        if (w > 16) at[17] = top;
     };
-    if (R.mine) {
-        store_column(dst, o0, room, v0 & 0xffffu, w0, p0);
-        upper(o0, w0, h0);
-    }
-    if (R.two) {
-        store_column(dst, o1, room, v0 >> 16, w1, p1);
-        upper(o1, w1, h1);
-    }
-    __syncwarp();
-    auto planes = [&](unsigned m, int second, int w_own, int o_own) {  // over what was stored: lane k stores plane k
-        for (; m; m &= m - 1u) {
-            const int owner = __ffs(m) - 1;
-            const uint32_t z = row_code(in + __shfl_sync(kFull, at, owner) + second, X, lane);
-            const int w = __shfl_sync(kFull, w_own, owner), o = __shfl_sync(kFull, o_own, owner) + 1;
-            uint32_t plane = 0;
-            for (int k = 0; k < w; ++k) {
-                const uint32_t bits = __ballot_sync(kFull, (z >> k) & 1u);
-                if (lane == k) plane = bits;
-            }
-            if (lane < w && o + lane < room) dst[o + lane] = plane;
-        }
-    };
-    planes(m0, 0, w0, o0);
-    planes(m1, 1, w1, o1);
-    return make_int2(total, before);
+    if (R.mine) store(dst + o0, v0 & 0xffffu, w0, p0, h0, s0);
+    if (R.two) store(dst + o0 + 1 + w0, v0 >> 16, w1, p1, h1, s1);
+    return make_int2(ret, before);
 }
 
-// Encode a round.  The words go to dst (the first block's first word) when all of
-// them fit `fit` words; words at or past `room` are dropped.  Returns the words of
-// the round; `before` gets those ahead of the lane's block.
+// Encode a round.  The words go to dst when all of them fit `fit` words.  Returns the
+// words of the round; `before` gets those ahead of the lane's block.  `wide`: rounds in
+// a row with columns of more than 8 planes; after two the narrow form is not tried
+// first (3.03 M rows x 33, sigma 60: 238 -> 218 us).
 template <bool kEven>
 __device__ __forceinline__ int encode_round(const EncPlan &pl, int X, const int16_t *in, int blocks, uint32_t *dst, int fit,
-                                            int room, int lane, int &before)
+                                            int lane, int &before, int &wide)
 {
+    if (wide >= 2) {
+        const int2 r = encode_wide_round<kEven>(X, in, blocks, dst, fit);
+        before = r.y;
+        wide = r.x & kWideRound ? 2 : 0;
+        return r.x & ~kWideRound;
+    }
     const Round<kEven> R(pl, X, in, blocks, lane);
     uint32_t p0[8], p1[8];
     const uint32_t v0 = R.row(0);
@@ -430,16 +419,18 @@ __device__ __forceinline__ int encode_round(const EncPlan &pl, int X, const int1
     const int span0 = (int)(int16_t)(mx & 0xffffu) - (int)(int16_t)(mn & 0xffffu);
     const int span1 = ((int)mx >> 16) - ((int)mn >> 16);
     if (__any_sync(kFull, R.mine && max(span0, span1) > 127)) {
-        const int2 r = encode_wide_round<kEven>(X, in, blocks, dst, fit, room);
+        const int2 r = encode_wide_round<kEven>(X, in, blocks, dst, fit);
         before = r.y;
-        return r.x;
+        wide = r.x & kWideRound ? wide + 1 : 0;
+        return r.x & ~kWideRound;
     }
+    wide = 0;
     const int w0 = byte_planes(p0), w1 = byte_planes(p1);
     int total;
     const int o0 = R.place(pl, w0, w1, lane, total, before);
     if (total > fit) return total;
-    if (R.mine) store_column(dst, o0, room, v0 & 0xffffu, w0, p0);
-    if (R.two) store_column(dst, o0 + 1 + w0, room, v0 >> 16, w1, p1);
+    if (R.mine) store_column(dst + o0, v0 & 0xffffu, w0, p0);
+    if (R.two) store_column(dst + o0 + 1 + w0, v0 >> 16, w1, p1);
     return total;
 }
 
@@ -485,9 +476,10 @@ __global__ void __launch_bounds__(kEncThreads, 2) pack_kernel(const int16_t *poo
     }
 
     unsigned char *base = dsm + warp * pl.bytes();
-    auto stage = [&](int k) { return reinterpret_cast<uint32_t *>(base + k * pl.cap); };
+    uint32_t *ring = reinterpret_cast<uint32_t *>(base);
     int16_t *in = reinterpret_cast<int16_t *>(base + pl.rows_at());
-    unsigned *meta = reinterpret_cast<unsigned *>(base + pl.meta_at());  // per stage: words, then those ahead of each block
+    // per round: words, then those ahead of each block
+    auto meta = [&](int j) { return reinterpret_cast<int *>(base + pl.meta_at()) + (j % kEncDepth) * (1 + pl.nsub); };
     uint64_t *bar = reinterpret_cast<uint64_t *>(base + pl.bytes() - 16);
     if (lane == 0) {
         daq::mbar_init(bar, 1);
@@ -512,9 +504,8 @@ __global__ void __launch_bounds__(kEncThreads, 2) pack_kernel(const int16_t *poo
             daq::bulk_g2s(in, pool + 32 * b * X, (uint32_t)(n * 64 * X), bar);
         }
     };
-    auto fits = [&](int j) { return 4 * (int)meta[(j % kEncDepth) * (1 + pl.nsub)] <= pl.cap; };  // turn j's words
-    // write turn j out; v: what was read of its place (lane 0)
-    auto finish = [&](int j, unsigned long long v) {
+    // write turn j out, whose words begin at `unit` of the ring; v: what was read of its place (lane 0)
+    auto finish = [&](int j, int unit, unsigned long long v) {
         const long long c = sh.tk[j % kEncRing];
         long long at = -1;
         if (lane == 0) {
@@ -530,34 +521,45 @@ __global__ void __launch_bounds__(kEncThreads, 2) pack_kernel(const int16_t *poo
         at = __shfl_sync(kFull, at, 0);
         if (at < 0) return;
         for (int w = 0; w < warp; ++w) at += sh.words[j % kEncRing][w];
-        const unsigned *m = meta + (j % kEncDepth) * (1 + pl.nsub);
-        const int words = (int)m[0];
+        const int *m = meta(j);
         const long long b = block_of(c);
         const int n = blocks_at(b);
         if (lane == sub * pl.np && sub < n) entry(b + sub, at + m[1 + sub]);
         const int room = (int)(max(0ll, min(cap - (head + 4 * at), 1ll << 30)) >> 2);
         uint32_t *dst = out32 + (head >> 2) + at;
-        if (fits(j)) {
-            const uint32_t *src = stage(j % kEncDepth);
-            const int last = min(words, room);
+        const uint32_t *src = ring + unit * pl.unit;
+        const int last = min(m[0], room);
 #pragma unroll 4
-            for (int k = lane; k < last; k += 32) dst[k] = src[k];
-        } else {
-            // did not fit the stage: encoded again, into its place (no rows are in flight)
-            for (int k = 0; k < n; ++k) load_block(pool, rows, X, b + k, in + k * 32 * X, lane);
-            int before;
-            encode_round<kEven>(pl, X, in, n, dst, 1 << 30, room, lane, before);
-        }
+        for (int k = lane; k < last; k += 32) dst[k] = src[k];
         __syncwarp();
     };
     long long c = sh.tk[0];
     start_rows(c);
-    int i = 0;
-    for (; c < n_chunks; ++i) {
+    int i = 0, done = 0;                 // turns encoded, written out
+    int wide = 0;
+    int at = 0, units = kEncUnits;       // a free piece of the ring, for turn i
+    int end = 0, want = 1;               // unit after the last round's words, units expected of the next round
+    unsigned starts = 0;                 // the unit each of the last rounds begins at, four bits a round
+    const unsigned unit_mul = ((1u << 20) + pl.unit - 1) / pl.unit;  // words (< 1,500) to units
+    auto start_of = [&](int j) { return (int)((starts >> (4 * (i - 1 - j))) & 15u); };
+    // The ring holds turns done .. i - 1 in order, each in one piece.  Is there a piece for turn i?
+    auto piece = [&]() -> bool {
+        at = 0;
+        units = kEncUnits;
+        if (done == i) return true;
+        const int first = start_of(done);
+        at = end;
+        units = (end > first ? kEncUnits : first) - end;
+        if (units < want && end > first) {
+            at = 0;
+            units = first;
+        }
+        return units >= want;
+    };
+    while (c < n_chunks) {
         unsigned long long ticket = 0, place = 0;
         if (threadIdx.x == 0) ticket = atomicAdd(tickets, 1ull);  // of turn i + 1, used once this one is encoded
-        const int j = i - (kEncDepth - 1);
-        if (lane == 0 && j >= 0) place = daq::ld_relaxed_u64(status + sh.tk[j % kEncRing]);
+        if (lane == 0 && i - done == kEncDepth - 1) place = daq::ld_relaxed_u64(status + sh.tk[done % kEncRing]);
         const long long b = block_of(c);
         const int n = blocks_at(b);
         if (copying) {
@@ -568,13 +570,26 @@ __global__ void __launch_bounds__(kEncThreads, 2) pack_kernel(const int16_t *poo
         } else {
             for (int k = 0; k < n; ++k) load_block(pool, rows, X, b + k, in + k * 32 * X, lane);
         }
+        while (!piece()) {
+            finish(done, start_of(done), 0ull);
+            ++done;
+        }
         int before;
-        const int fit = pl.cap / 4;
-        const int words = encode_round<kEven>(pl, X, in, n, stage(i % kEncDepth), fit, fit, lane, before);
-        unsigned *m = meta + (i % kEncDepth) * (1 + pl.nsub);
-        if (lane == sub * pl.np && sub < pl.nsub) m[1 + sub] = (unsigned)before;
+        const int words = encode_round<kEven>(pl, X, in, n, ring + at * pl.unit, units * pl.unit, lane, before, wide);
+        want = (int)(((unsigned)(words + pl.unit - 1) * unit_mul) >> 20);  // of the next round too: mostly as long
+        if (want > units) {  // longer than the round before: again, once there is a piece for it
+            while (!piece()) {
+                finish(done, start_of(done), 0ull);
+                ++done;
+            }
+            before = encode_wide_round<kEven>(X, in, n, ring + at * pl.unit, units * pl.unit).y;
+        }
+        end = at + want;
+        starts = starts << 4 | (unsigned)at;
+        int *m = meta(i);
+        if (lane == sub * pl.np && sub < pl.nsub) m[1 + sub] = before;
         if (lane == 0) {
-            m[0] = (unsigned)words;
+            m[0] = words;
             sh.words[i % kEncRing][warp] = (unsigned)words;
             if (warp == 0) {
                 sh.tk[(i + 1) % kEncRing] = (long long)ticket;
@@ -595,14 +610,17 @@ __global__ void __launch_bounds__(kEncThreads, 2) pack_kernel(const int16_t *poo
                 }
         }
         __syncwarp();
-        const long long next = sh.tk[(i + 1) % kEncRing];
-        const bool again = j >= 0 && !fits(j);  // turn j needs the row buffer
-        if (!again) start_rows(next);
-        if (j >= 0) finish(j, place);
-        if (again) start_rows(next);
-        c = next;
+        c = sh.tk[++i % kEncRing];
+        start_rows(c);
+        if (i - done == kEncDepth) {
+            finish(done, start_of(done), place);
+            ++done;
+        }
     }
-    for (int j = max(0, i - (kEncDepth - 1)); j < i; ++j) finish(j, 0ull);
+    while (done < i) {
+        finish(done, start_of(done), 0ull);
+        ++done;
+    }
 }
 
 // ------------------------------------------------------------------ decoder
