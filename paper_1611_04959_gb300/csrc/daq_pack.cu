@@ -29,10 +29,6 @@ constexpr int kMaxX = 64;
 constexpr uint32_t kMagic = 0x50514144u;
 constexpr uint64_t kWaitNs = 4000000000ull;  // a block copy not landed, or an earlier chunk not heard of, after this: give up
 
-__device__ __forceinline__ uint32_t zigzag(int32_t d) { return ((uint32_t)d << 1) ^ (uint32_t)(d >> 31); }
-
-__device__ __forceinline__ int32_t unzigzag(uint32_t z) { return (z & 1u) ? -(int32_t)((z + 1u) >> 1) : (int32_t)(z >> 1); }
-
 // Copy block b's rows (16-byte vectors; the pool and every block start are
 // 16-byte aligned) into the warp's shared rows, rows past the pool's end
 // repeating its final row.  Returns the number of real rows.
@@ -642,8 +638,13 @@ __global__ void __launch_bounds__(kEncThreads, 2) pack_kernel(const int16_t *poo
 // group's payload is brought into L2 while this one is decoded (390 -> 383
 // us).  Undoing the zigzag on bytes after the swaps, copying rows out with
 // 16-byte stores and checking every head word in the walk took 502 us.
-// Columns wider than 8 bits (pulses: 2% of the blocks of a dense fill hold some)
-// are then done again by the whole warp, lanes on rows.
+// Where one of a warp's columns is wider than 8 bits (pulses: 2% of the blocks of a
+// dense fill hold some) all take the same way with 16-bit differences, low and high
+// bytes: 2 M rows x 54 take 62 us at sigma 3, 86 at 24, 102 at 60, 132 full-range.
+// (Such columns done again one at a time by the whole warp, lanes on rows: 62, 80, 585
+// and 808; lanes on rows throughout: 206, 500, 510 and 549.  That loop kept for up to
+// three columns: 64 at sigma 3, 82 at 24.  The wide form as a function: 63 and 86, and
+// 6% more than this for odd crystal counts, whose registers the call spills.)
 constexpr int kDecWarps = 4;
 constexpr int kDecThreads = 32 * kDecWarps;
 
@@ -673,6 +674,49 @@ __device__ __forceinline__ void column_steps(const uint32_t *h, int w, uint32_t 
     for (int k = 0; k < 7; ++k) p[k] = (h[2 + k] & (uint32_t)((k + 1 - w) >> 31)) ^ sign;
     p[7] = sign;
     swap_bits8(p);
+}
+
+// The rows of a lane's two columns (head words at words + at0 and + at1, negative: it
+// has none) where one of the warp's is wider than 8 bits: the differences modulo 2^16,
+// as low and high bytes.  Their planes are planes 1 .. 16 of the codes, each xor the sign; a
+// sample is 16 bits too, so that the carry past them is of no account.
+template <bool kEven>
+__device__ __forceinline__ void decode_wide(const uint32_t *words, int at0, int at1, int16_t *o, int X)
+{
+    const bool mine = at0 >= 0, two = at1 >= 0;
+    const uint32_t *h0 = words + max(at0, 0), *h1 = words + max(at1, 0);
+    uint32_t a0 = mine ? h0[0] : 0u, a1 = two ? h1[0] : 0u, b0 = 0, b1 = 0;  // sample = a + 256 b, modulo 2^16
+    auto steps = [](const uint32_t *h, int w, uint32_t (&lo)[8], uint32_t (&hi)[8]) {
+        const uint32_t sign = h[1] & (uint32_t)(-w >> 31);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            lo[k] = (h[2 + k] & (uint32_t)((k + 1 - w) >> 31)) ^ sign;
+            hi[k] = (h[10 + k] & (uint32_t)((k + 9 - w) >> 31)) ^ sign;
+        }
+        swap_bits8(lo);
+        swap_bits8(hi);
+    };
+    uint32_t lo0[8], hi0[8], lo1[8], hi1[8];
+    steps(h0, (int)(a0 >> 16), lo0, hi0);
+    steps(h1, (int)(a1 >> 16), lo1, hi1);
+    if (!mine) return;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+        const int k = q & 7, j = q >> 3;
+        if (q) {
+            a0 = __dp4a(lo0[k], 1u << (8 * j), a0);
+            b0 = __dp4a(hi0[k], 1u << (8 * j), b0);
+            a1 = __dp4a(lo1[k], 1u << (8 * j), a1);
+            b1 = __dp4a(hi1[k], 1u << (8 * j), b1);
+        }
+        const uint32_t s0 = a0 + (b0 << 8), s1 = a1 + (b1 << 8);
+        if (kEven) {
+            *reinterpret_cast<uint32_t *>(o + q * X) = __byte_perm(s0, s1, 0x5410);
+        } else {
+            o[q * X] = (int16_t)s0;
+            if (two) o[q * X + 1] = (int16_t)s1;
+        }
+    }
 }
 
 template <bool kEven>
@@ -707,27 +751,6 @@ __global__ void __launch_bounds__(kDecThreads, 5) unpack_kernel(const unsigned c
     auto bulk_read_done = [&] {
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         __syncwarp();
-    };
-    // columns wider than 8 bits (owner lanes m, head words at h, first rows at o),
-    // one at a time by the whole warp, lanes on rows
-    auto wide_columns = [&](unsigned m, const uint32_t *h, int16_t *o) {
-        const uint32_t *words = reinterpret_cast<const uint32_t *>(base);
-        const int hw = (int)(h - words), oe = (int)(o - out);
-        for (; m; m &= m - 1u) {
-            const int owner = __ffs(m) - 1;
-            const uint32_t *hc = words + __shfl_sync(kFull, hw, owner);
-            int16_t *oc = out + __shfl_sync(kFull, oe, owner);
-            const int w = (int)(hc[0] >> 16);
-            uint32_t z = 0;
-            for (int k = 0; k < w; ++k) z |= ((hc[1 + k] >> lane) & 1u) << k;
-            int32_t d = lane ? unzigzag(z) : 0;
-#pragma unroll
-            for (int s = 1; s < 32; s <<= 1) {
-                const int32_t y = __shfl_up_sync(kFull, d, s);
-                if (lane >= s) d += y;
-            }
-            oc[lane * X] = (int16_t)((int32_t)(int16_t)(hc[0] & 0xffffu) + d);
-        }
     };
     auto offset_of = [&](long long b) { return lane <= pl.G && b + lane <= nb ? offs[b + lane] : ~0ull; };
     unsigned long long next_off = b0 < nb ? offset_of(b0) : 0ull;
@@ -828,30 +851,32 @@ __global__ void __launch_bounds__(kDecThreads, 5) unpack_kernel(const unsigned c
                 const uint32_t v0 = mine ? h0[0] : 0u, v1 = two ? h1[0] : 0u;
                 const int w0 = (int)(v0 >> 16), w1 = (int)(v1 >> 16);
                 int16_t *o = out + (sub < pl.nsub ? sub : 0) * 32 * X + x0;
-                uint32_t p0[8], p1[8];
-                column_steps(h0, w0, p0);
-                column_steps(h1, w1, p1);
-                bulk_read_done();
-                int32_t a0 = (int32_t)v0, a1 = (int32_t)v1;  // the low halves count
-                if (mine) {
+                if (__any_sync(kFull, max(w0, w1) > 8)) {
+                    bulk_read_done();
+                    decode_wide<kEven>(words, mine ? (int)(h0 - words) : -1, two ? (int)(h1 - words) : -1, o, X);
+                } else {
+                    uint32_t p0[8], p1[8];
+                    column_steps(h0, w0, p0);
+                    column_steps(h1, w1, p1);
+                    bulk_read_done();
+                    int32_t a0 = (int32_t)v0, a1 = (int32_t)v1;  // the low halves count
+                    if (mine) {
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) {
-                        const int k = q & 7, j = q >> 3;
-                        if (q) {
-                            a0 = __dp4a((int)p0[k], 1 << (8 * j), a0);
-                            a1 = __dp4a((int)p1[k], 1 << (8 * j), a1);
-                        }
-                        if (kEven) {
-                            *reinterpret_cast<uint32_t *>(o + q * X) = __byte_perm((uint32_t)a0, (uint32_t)a1, 0x5410);
-                        } else {
-                            o[q * X] = (int16_t)a0;
-                            if (two) o[q * X + 1] = (int16_t)a1;
+                        for (int q = 0; q < 32; ++q) {
+                            const int k = q & 7, j = q >> 3;
+                            if (q) {
+                                a0 = __dp4a((int)p0[k], 1 << (8 * j), a0);
+                                a1 = __dp4a((int)p1[k], 1 << (8 * j), a1);
+                            }
+                            if (kEven) {
+                                *reinterpret_cast<uint32_t *>(o + q * X) = __byte_perm((uint32_t)a0, (uint32_t)a1, 0x5410);
+                            } else {
+                                o[q * X] = (int16_t)a0;
+                                if (two) o[q * X + 1] = (int16_t)a1;
+                            }
                         }
                     }
                 }
-                __syncwarp();
-                wide_columns(__ballot_sync(kFull, w0 > 8), h0, o);
-                wide_columns(__ballot_sync(kFull, w1 > 8), h1, o + 1);
                 __syncwarp();
                 // rows of the good blocks to the pool: a bulk copy per whole block
                 const bool whole = 32 * (b0 + g0 + r + pl.nsub) <= rows;
