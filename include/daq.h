@@ -178,11 +178,13 @@ typedef struct daq_island {
  *   wait_limit_ns  limit of each device-side wait on state that other CTAs
  *                publish (0 = 4 s): the look-back over earlier tiles (every
  *                form's scan), the single-launch form's scanner and lag
- *                waits, and the phased form's wait for a chunk's aggregates.  A wait that runs out sets DAQ_DEV_TIMEOUT; every CTA
- *                then stops taking work, waits for its own copies in flight
- *                and exits, and the call returns DAQ_ETIMEOUT with incomplete
+ *                waits, and the phased form's wait for a chunk's aggregates.
+ *                A wait that runs out sets DAQ_DEV_TIMEOUT; every CTA then
+ *                stops taking work, waits for its own copies in flight and
+ *                exits, and the call returns DAQ_ETIMEOUT with incomplete
  *                outputs.  The next call starts clean.  Waits of a CTA on its
- *                own warps keep the 4 s limit.
+ *                own warps have 4 s, in the single-launch and the phased form
+ *                on top of this limit: they may wait for other CTAs in turn.
  */
 typedef struct daq_params {
     int32_t threshold;

@@ -1212,6 +1212,7 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     a.calo_base = p.calo_base;
     a.q_calos = (int32_t)q_calos;
     a.wait_ns = p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs;
+    a.own_wait_ns = a.wait_ns > UINT64_MAX - kWaitLimitNs ? UINT64_MAX : a.wait_ns + kWaitLimitNs;
     a.fill_len = p.fill_len;
     a.flags = p.flags;
     auto geometry = [&] {

@@ -109,7 +109,8 @@ struct KArgs {
     int64_t qbins[2], qoff[2];
     int32_t fill_base, calo_base;
     int32_t q_calos;  // calorimeter rows of each decimation's block of Q
-    uint64_t wait_ns;  // limit of waits on other CTAs' published state
+    uint64_t wait_ns;      // limit of waits on other CTAs' published state
+    uint64_t own_wait_ns;  // of waits on the CTA's own warps where those wait for other CTAs
     const int32_t *fill_len;
     uint32_t flags;
     int32_t hl, hr, ew, rs;  // halo left/right, extended width, smem row pitch (bytes) = 2 boxw

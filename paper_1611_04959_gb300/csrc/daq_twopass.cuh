@@ -129,7 +129,9 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity)
 }
 
 // As warp_wait, but also giving up once a CTA has flagged a timeout (the
-// single-launch form, whose waits on other CTAs may run out).
+// single-launch and the phased form, whose waits on other CTAs may run out).  What
+// another warp of the CTA hands on may itself wait for other CTAs, so the limit is
+// a.own_wait_ns, which outlasts theirs.
 __device__ __forceinline__ bool warp_wait_abortable(const KArgs &a, uint64_t *bar, uint32_t parity)
 {
     bool ok = mbar_try_wait(bar, parity);
@@ -140,7 +142,7 @@ __device__ __forceinline__ bool warp_wait_abortable(const KArgs &a, uint64_t *ba
                 ok = true;
                 break;
             }
-            if ((i & 63u) == 0u && (aborted(a) || global_ns() - t0 > kWaitLimitNs)) break;
+            if ((i & 63u) == 0u && (aborted(a) || global_ns() - t0 > a.own_wait_ns)) break;
         }
     }
     return !__any_sync(kFull, !ok);
