@@ -409,10 +409,13 @@ __device__ __forceinline__ void count_role(const KArgs &a, unsigned char *smem, 
         }
         if (kRows) row_load_wait();  // a warp that stopped early has copies in flight
         // a warp that stopped early leaves loads in flight: they land before
-        // the CTA may exit (a slot's latest phase; immediate when consumed)
-        if (kFused && tid == 0)
+        // the CTA may exit (a slot's latest phase; immediate when consumed, and
+        // complete only with the record of the last load)
+        if (kFused && tid == 0) {
+            finish_load();
             for (int k = 0; k < NS; ++k)
                 if (pend & (1u << k)) mbar_wait_bounded(full + k, (pend_par >> k) & 1u, kWaitLimitNs);
+        }
     } else if (warp < NSW + NS) {
         // ------------------------------------------------------------ marks, aggregate, Q bins of buffer s
         const int s = warp - NSW;
