@@ -344,10 +344,25 @@ def daq_unpack_pool(in_ptr, in_bytes, rows, n_xtal, out_ptr, err_ptr, stream_ptr
     return int(lib().daq_unpack_pool(in_ptr, in_bytes, rows, n_xtal, out_ptr, err_ptr, stream_ptr))
 
 
-def pack_pool(pool, rows: int | None = None, stream=None, out=None, workspace=None):
-    """Pack the first `rows` rows of a CUDA int16 pool [rows][X].  Returns
-    (stream uint8 tensor view of its exact size, size)."""
+def _on(stream, device):
+    """Context in which allocations, calls and reads go to the caller's `stream`."""
     import torch
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(int(stream.cuda_stream), device=device)
+    return torch.cuda.stream(stream)
+
+
+def pack_pool(pool, rows: int | None = None, stream=None, out=None, workspace=None):
+    """Pack the first `rows` rows of a CUDA int16 pool [rows][X] on `stream`, which is
+    waited for.  Returns (stream uint8 tensor view of its exact size, size)."""
+    import torch
+    if stream is not None:
+        caller = torch.cuda.current_stream(pool.device)
+        with _on(stream, pool.device):
+            packed, n = pack_pool(pool, rows, None, out, workspace)
+        if out is None or packed.data_ptr() != out.data_ptr():
+            packed.record_stream(caller)
+        return packed, n
     rows = pool.shape[0] if rows is None else int(rows)
     X = int(pool.shape[1])
     dev = pool.device
@@ -358,7 +373,7 @@ def pack_pool(pool, rows: int | None = None, stream=None, out=None, workspace=No
     if workspace is None or workspace.numel() < need:
         workspace = torch.empty(need, dtype=torch.uint8, device=dev)
     nbytes = torch.empty(1, dtype=torch.int64, device=dev)   # always written by the call
-    stream = torch.cuda.current_stream(dev) if stream is None else stream
+    stream = torch.cuda.current_stream(dev)
     rc = daq_pack_pool(pool.data_ptr(), rows, X, out.data_ptr(), out.numel(), nbytes.data_ptr(), workspace.data_ptr(),
                        workspace.numel(), stream.cuda_stream)
     if rc != DAQ_OK:
@@ -368,12 +383,19 @@ def pack_pool(pool, rows: int | None = None, stream=None, out=None, workspace=No
 
 
 def unpack_pool(packed, rows: int, n_xtal: int, stream=None):
-    """Decode a packed stream (CUDA uint8 tensor) into a new int16 [rows][n_xtal] tensor."""
+    """Decode a packed stream (CUDA uint8 tensor) into a new int16 [rows][n_xtal] tensor
+    on `stream`, which is waited for."""
     import torch
     dev = packed.device
+    if stream is not None:
+        caller = torch.cuda.current_stream(dev)
+        with _on(stream, dev):
+            out = unpack_pool(packed, rows, n_xtal)
+        out.record_stream(caller)
+        return out
     out = torch.empty((max(1, rows), n_xtal), dtype=torch.int16, device=dev)
     err = torch.empty(1, dtype=torch.int32, device=dev)      # the call clears it
-    stream = torch.cuda.current_stream(dev) if stream is None else stream
+    stream = torch.cuda.current_stream(dev)
     rc = daq_unpack_pool(packed.data_ptr(), packed.numel(), rows, n_xtal, out.data_ptr(), err.data_ptr(),
                          stream.cuda_stream)
     if rc != DAQ_OK:
