@@ -642,7 +642,9 @@ int daq_crystal_sum(const int16_t *samples, int n_calo, int n_xtal, int64_t n_sa
  *                         so out_cap >= daq_pack_bound() is always enough -
  *                         or -1 when a device-side wait (for a copy of pool
  *                         rows, or for the sizes of earlier blocks) ran out
- *                         after 4 s (the stream is then not valid).
+ *                         after 4 s (the stream is then not valid).  Other
+ *                         work that keeps the call's CTAs from starting only
+ *                         delays it, up to 60 s.
  * daq_unpack_pool         decode a stream of in_bytes bytes into device
  *                         pool_out[rows][n_xtal]; *err (device int32) is set
  *                         to 0, or to a non-zero code when the header does not

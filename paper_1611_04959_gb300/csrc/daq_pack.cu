@@ -28,6 +28,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxX = 64;
 constexpr uint32_t kMagic = 0x50514144u;
 constexpr uint64_t kWaitNs = 4000000000ull;  // a block copy not landed, or an earlier chunk not heard of, after this: give up
+constexpr uint64_t kStartNs = 60000000000ull;  // no CTA has taken the next chunk after this: give up
 
 // Copy block b's rows (16-byte vectors; the pool and every block start are
 // 16-byte aligned) into the warp's shared rows, rows past the pool's end
@@ -180,14 +181,15 @@ __device__ __forceinline__ void st_release_cta(int *p, int v)
 // The scanning CTA: turns the published sizes of chunks 0, 1, ... into places.
 // Each round reads the next 2 kEncThreads words and takes those before the first
 // that is not there yet.  Returns the payload's words, -1 when it gave up: the
-// chunks that had not got a place are then told so.
-__device__ long long enc_places(unsigned long long *st, long long n_chunks)
+// chunks that had not got a place are then told so.  A chunk that no CTA has taken
+// (`tickets`: chunks taken) is not late: other work may hold all SMs but this CTA's.
+__device__ long long enc_places(unsigned long long *st, long long n_chunks, const unsigned long long *tickets)
 {
     __shared__ unsigned s_sum[kEncWarps], s_miss[kEncWarps];
     __shared__ int s_stop;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     long long done = 0, at = 0;
-    uint64_t t0 = daq::global_ns();
+    uint64_t t0 = daq::global_ns(), t_last = t0;  // of the next chunk's wait, of the last chunk placed
     if (tid == 0) s_stop = 0;
     __syncthreads();
     while (done < n_chunks) {
@@ -215,8 +217,11 @@ __device__ long long enc_places(unsigned long long *st, long long n_chunks)
             if (w < warp) ahead += s_sum[w];
         }
         const uint64_t now = daq::global_ns();
-        if (first > 0) t0 = now;
-        if (tid == 0 && now - t0 > kWaitNs) s_stop = 1;
+        if (first > 0) t0 = t_last = now;
+        if (tid == 0 && now - t0 > kWaitNs / 2) {
+            if (daq::ld_relaxed_u64(tickets) <= (unsigned long long)done) t0 = now;
+            if (now - t0 > kWaitNs || now - t_last > kStartNs) s_stop = 1;
+        }
         // words before this thread's pair; of them only those before `first` count, and every pair before it is whole
         const long long mine = at + ahead + incl - a - b;
         if (2 * tid < (int)first) daq::st_relaxed_u64(st + done + 2 * tid, ((unsigned long long)mine << 2) | kIncl);
@@ -463,7 +468,7 @@ __global__ void __launch_bounds__(kEncThreads, 2) pack_kernel(const int16_t *poo
             out32[1] = (uint32_t)X;
             reinterpret_cast<unsigned long long *>(out)[1] = (unsigned long long)rows;
         }
-        const long long words = enc_places(status, n_chunks);
+        const long long words = enc_places(status, n_chunks, tickets);
         if (threadIdx.x == 0) {
             if (words >= 0) entry(nb, words);
             *out_bytes = words >= 0 ? head + 4 * words : -1ll;
