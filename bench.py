@@ -279,7 +279,7 @@ def bench_gb300(args, ws, rank, local):
             call(p, ctypes.cast(ev_arrays[k], ctypes.c_void_p).value)
     torch.cuda.synchronize(dev)
     step_ms = [e[0].elapsed_time(e[4]) for e in evs]
-    kern = kernel_means(evs)
+    kern = kernel_means(evs, form_kernels(daq, daq.daq_call_form(samples.data_ptr(), C, X, N, F, p)))
     _, elapsed_ms, value = replicas.aggregate(K * raw_bytes, elapsed_ms, dev)
 
     # ---- roofline of the dominant kernel: the phased kernel (reads the samples once from HBM, adds to Q,
@@ -548,8 +548,8 @@ def bench_batched(args, torch, dev, daq, synth, W, w=None, plain_flags=0) -> dic
              "form": "default kernels, one daq_process_fills call per fill (16 calls per batch), "
                      "no graph, no tuning" + (f", flags {plain_flags}" if plain_flags else "")}
     del ws1
-    # prepare and phased kernel, or prepare, count, scan and compact
-    per_batch = 2 if tuning["grid"] == 0 and tuning["tile"] in (0, 448) and not tuning.get("flags", 0) & daq.DAQ_SPARSE else 4
+    tuned = daq.make_params(**params, tile=tuning["tile"], grid=tuning["grid"], flags=tuning.get("flags", 0))
+    per_batch = len(form_kernels(daq, daq.daq_call_form(samples.data_ptr(), C, X, N, F, tuned)))
     res = {"value": round(Kb * raw / (total_ms * 1e-3) / 1e9, 2), "unit": UNIT, "steps": Kb,
            "ms_per_batch": round(total_ms / Kb, 4),
            "latency_ms": {"p50": round(statistics.median(ms), 4), "p99": round(float(np.percentile(ms, 99)), 4)},
@@ -618,14 +618,19 @@ def copy_bandwidth(torch, dev, host_in, dev_in, host_out, dev_out, out_rows: int
                       "(d2h), alone and concurrently on two streams"}
 
 
-def kernel_means(evs) -> dict:
-    """Mean ms of each kernel of a call from its DAQ_N_EVENTS events per step.  The
-    phased form records the last three after its one kernel, so nothing lies
-    between them (a compact kernel takes longer than a few microseconds)."""
+def form_kernels(daq, form: int, skip_islands: bool = False) -> list:
+    """The kernels that a call of this form launches, in order."""
+    if form == daq.DAQ_FORM_PHASED:
+        return ["daq_prepare_kernel", "daq_phase_kernel"]
+    if form == daq.DAQ_FORM_TWO_PASS:
+        return ["daq_prepare_kernel", "daq_count_kernel", "daq_scan_kernel"] + ([] if skip_islands else ["daq_compact_kernel"])
+    return ["daq_prepare_kernel", "daq_tile_kernel"]
+
+
+def kernel_means(evs, names) -> dict:
+    """Mean ms of each kernel of a call (`names`: form_kernels) from its DAQ_N_EVENTS events
+    per step."""
     mean = [statistics.fmean(r[i].elapsed_time(r[i + 1]) for r in evs) for i in range(4)]
-    names = ["daq_prepare_kernel", "daq_count_kernel", "daq_scan_kernel", "daq_compact_kernel"]
-    if mean[3] < 0.004:
-        names = ["daq_prepare_kernel", "daq_phase_kernel"]
     return {name: round(ms, 4) for name, ms in zip(names, mean)}
 
 
@@ -668,7 +673,8 @@ def time_calls(torch, dev, daq, x, F, C, X, N, params, K: int, out=None, warm: i
     p.events = None
     torch.cuda.synchronize(dev)
     ms = [r[0].elapsed_time(r[4]) for r in evs]
-    kern = kernel_means(evs)
+    names = form_kernels(daq, daq.daq_call_form(x.data_ptr(), C, X, N, F, p), bool(p.flags & daq.DAQ_SKIP_ISLANDS))
+    kern = kernel_means(evs, names)
     counts = out.counts.cpu().numpy()
     del ws, q
     return total, ms, kern, counts

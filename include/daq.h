@@ -279,6 +279,23 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
                       const daq_params *params, const daq_islands *islands_out, int64_t *qhist_inout);
 
 /*
+ * The form (DAQ_FORM_*) that daq_process_fills takes for such a call on the current
+ * device, or a negative status.  A device that refuses the phased form's cooperative
+ * launch, or a tensor map, runs the two-pass form instead.
+ */
+enum daq_form {
+    DAQ_FORM_TWO_PASS = 0,      /* count kernel, scan, compact kernel */
+    DAQ_FORM_PLAIN = 1,         /* grid -1, -2 */
+    DAQ_FORM_PIPELINED = 2,     /* grid -3 */
+    DAQ_FORM_SINGLE_LAUNCH = 3, /* grid -4 */
+    DAQ_FORM_STREAM = 4,        /* grid -5 */
+    DAQ_FORM_SINGLE_READ = 5,   /* grid -6 */
+    DAQ_FORM_PHASED = 6
+};
+int daq_call_form(const int16_t *samples, int n_calo, int n_xtal, int64_t n_samples, int n_fills,
+                  const daq_params *params);
+
+/*
  * Wait for everything queued on `stream` so far, copy a call's counts[4] to host
  * memory and return the call's status (as DAQ_SYNC does, for callers that want the
  * counts too): one wait for both.  DAQ_EINVAL for a null pointer.

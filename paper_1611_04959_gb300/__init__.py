@@ -24,6 +24,9 @@ DAQ_STATIC_SCRATCH_BYTES = 8 << 20
 DAQ_SKIP_Q, DAQ_SKIP_ISLANDS, DAQ_SYNC, DAQ_PACK_POOL, DAQ_DEBUG_CHECKS, DAQ_SPARSE = 1, 2, 4, 8, 16, 32
 DAQ_DEV_HDR_OVERFLOW, DAQ_DEV_POOL_OVERFLOW, DAQ_DEV_TIMEOUT, DAQ_DEV_BAD_FILL_LEN, DAQ_DEV_BAD_INDEX = 1, 2, 4, 8, 16
 
+(DAQ_FORM_TWO_PASS, DAQ_FORM_PLAIN, DAQ_FORM_PIPELINED, DAQ_FORM_SINGLE_LAUNCH, DAQ_FORM_STREAM, DAQ_FORM_SINGLE_READ,
+ DAQ_FORM_PHASED) = range(7)
+
 ISLAND_DTYPE = np.dtype([("fill", "<i4"), ("calo", "<i4"), ("start", "<i4"), ("len", "<i4"),
                          ("pool_row", "<i8")])
 
@@ -134,6 +137,8 @@ def lib():
             L.daq_process_fills_host.restype = i32
             L.daq_trace_tiles.argtypes = [i32, i32, i64, i32, ctypes.POINTER(DaqParams)]
             L.daq_trace_tiles.restype = i64
+            L.daq_call_form.argtypes = [vp, i32, i32, i64, i32, ctypes.POINTER(DaqParams)]
+            L.daq_call_form.restype = i32
             L.daq_read_counts.argtypes = [vp, vp, vp]
             L.daq_read_counts.restype = i32
             L.daq_status_from_counts.argtypes = [vp]
@@ -235,6 +240,11 @@ def daq_process_fills(samples_ptr: int, n_calo: int, n_xtal: int, n_samples: int
                       params: DaqParams, islands: DaqIslands, qhist_ptr: int | None) -> int:
     return int(lib().daq_process_fills(samples_ptr, n_calo, n_xtal, n_samples, n_fills, ctypes.byref(params),
                                        ctypes.byref(islands), qhist_ptr))
+
+
+def daq_call_form(samples_ptr: int, n_calo: int, n_xtal: int, n_samples: int, n_fills: int, params: DaqParams) -> int:
+    """DAQ_FORM_* that daq_process_fills takes for such a call, or a negative status."""
+    return int(lib().daq_call_form(samples_ptr, n_calo, n_xtal, n_samples, n_fills, ctypes.byref(params)))
 
 
 def daq_read_counts(counts_ptr: int, counts_host: np.ndarray, stream=None) -> int:

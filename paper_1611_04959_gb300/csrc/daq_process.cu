@@ -1036,6 +1036,31 @@ static bool phase_geometry(Plan *pl, int pre, int post, int X)
     return true;
 }
 
+// Rows that the tensor boxes take: 16-byte aligned, all of them.
+static bool rows_aligned(const int16_t *samples, int64_t total, int64_t n_samples)
+{
+    return total > 0 && n_samples % 8 == 0 && (reinterpret_cast<uintptr_t>(samples) & 15) == 0;
+}
+
+// The default form is phased where it can be and pays: whole tiles of 448 samples
+// loaded by boxes, islands written, a plan that fits in shared memory, enough tiles an SM.  Not
+// with DAQ_SPARSE, whose compact kernel skips what this form would still step
+// through (313 us against 326 with a fifth of the nominal pulse rate, 356 / 337 at the
+// nominal rate), nor for a caller's own short limit on waits, which are longer here (a
+// CTA waits for the slowest of a chunk), nor under a trace.  *pl: the two-pass plan,
+// replaced where the call takes the phased form.
+static bool take_phased(const daq_params &p, bool aligned, int n_xtal, int n_fills, const DeviceInfo &di, Plan *pl)
+{
+    if (p.grid != 0 || !aligned || (p.flags & (DAQ_SKIP_ISLANDS | DAQ_SPARSE)) || p.trace || n_fills > kPlanSmem ||
+        (p.wait_limit_ns != 0 && p.wait_limit_ns < kPhaseMinWaitNs) ||
+        pl->max_tiles < (int64_t)phase_min_tiles(*pl, n_xtal) * di.sms)
+        return false;
+    Plan r = *pl;
+    if (!phase_geometry(&r, p.pre, p.post, n_xtal) || (int)r.smem > di.smem_optin) return false;
+    *pl = r;
+    return true;
+}
+
 // Phased form: one cooperative launch, one CTA per SM.
 template <int kWin, bool kPlain>
 static cudaError_t launch_phase(const KArgs &a, const Plan &pl, int sms, cudaStream_t s)
@@ -1240,7 +1265,7 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
     if (cudaGetDevice(&dev) != cudaSuccess) return DAQ_ECUDA;
     const DeviceInfo di = device_info(dev);
     if (di.sms <= 0) return DAQ_ECUDA;
-    const bool aligned = total > 0 && n_samples % 8 == 0 && (reinterpret_cast<uintptr_t>(samples) & 15) == 0;
+    const bool aligned = rows_aligned(samples, total, n_samples);
     auto encode_maps = [&] {
         a.use_tma = aligned &&
                     encode_tensor_map(&a.tmap, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples, pl.boxw,
@@ -1248,19 +1273,8 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
                     encode_tensor_map(&a.tmap_b, samples, (int64_t)n_fills * n_calo * n_xtal, n_samples,
                                       pl.boxw_b, n_xtal);
     };
-    // The default form is phased where it can be and pays: whole tiles of 448 samples
-    // loaded by boxes, islands written, a plan that fits in shared memory, enough tiles an SM.  Not
-    // with DAQ_SPARSE, whose compact kernel skips what this form would still step
-    // through (313 us against 326 with a fifth of the nominal pulse rate, 356 / 337 at the
-    // nominal rate), nor for a caller's own short limit on waits, which are longer here (a
-    // CTA waits for the slowest of a chunk), nor under a trace.
     const Plan twopass = pl;
-    if (p.grid == 0 && aligned && !skip_isl && !(p.flags & DAQ_SPARSE) && !p.trace && n_fills <= kPlanSmem &&
-        (p.wait_limit_ns == 0 || p.wait_limit_ns >= kPhaseMinWaitNs) &&
-        pl.max_tiles >= (int64_t)phase_min_tiles(pl, n_xtal) * di.sms) {
-        if (phase_geometry(&pl, p.pre, p.post, n_xtal) && (int)pl.smem <= di.smem_optin) geometry();
-        else pl = twopass;
-    }
+    if (take_phased(p, aligned, n_xtal, n_fills, di, &pl)) geometry();
     encode_maps();
     auto take_twopass = [&] {
         pl = twopass;
@@ -1401,6 +1415,21 @@ int daq_process_fills(const int16_t *samples, int n_calo, int n_xtal, int64_t n_
         return daq_read_counts(out->counts, h, p.stream);
     }
     return DAQ_OK;
+}
+
+int daq_call_form(const int16_t *samples, int n_calo, int n_xtal, int64_t n_samples, int n_fills, const daq_params *params)
+{
+    Plan pl;
+    const int rc = make_plan(n_calo, n_xtal, n_samples, n_fills, params, &pl);
+    if (rc) return rc;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return DAQ_ECUDA;
+    const DeviceInfo di = device_info(dev);
+    if (di.sms <= 0) return DAQ_ECUDA;
+    const bool aligned = rows_aligned(samples, (int64_t)n_fills * n_calo * n_xtal * n_samples, n_samples);
+    if ((pl.mode == kModeStream && !aligned) || (pl.mode == kModePark && (!aligned || (n_xtal & 1)))) return kModeTwoPass;
+    take_phased(*params, aligned, n_xtal, n_fills, di, &pl);
+    return pl.mode;
 }
 
 // One wait: the copy is queued behind the call and the stream waited for once.  (A

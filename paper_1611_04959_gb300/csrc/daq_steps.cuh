@@ -21,7 +21,7 @@ namespace daq {
 
 constexpr uint64_t kWaitLimitNs = 4000000000ull;  // bounded device waits (4 s)
 constexpr int kMaxTileWords = 14;                 // marks words of the widest two-pass tile (448 samples)
-// kernels a call may use (daq_params.grid picks one)
+// kernels a call may use (daq_params.grid picks one): the DAQ_FORM_ codes
 enum : int32_t { kModeTwoPass = 0, kModePlain = 1, kModePipelined = 2, kModeFused = 3, kModeStream = 4, kModePark = 5, kModePhased = 6 };
 // daq_params-independent choice of the tile loads: element by element, tensor
 // boxes, or (two-pass form, rows that share no 16-byte alignment) row by row
