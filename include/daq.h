@@ -133,7 +133,13 @@ typedef struct daq_island {
  *                     and 14 tiles an SM (2 where the windows are wide:
  *                     post = 64, 48 crystals);
  *                     a caller confined to some of the SMs gets the two-pass
- *                     form;
+ *                     form.  Its CTAs start together, one on every SM, and
+ *                     take nearly all of an SM's shared memory: it waits for
+ *                     long-lived kernels of other streams, and the kernels of
+ *                     such calls on several streams follow one another.  A
+ *                     caller whose call must run beside a kernel that holds
+ *                     SMs asks for the two-pass form with grid > 0.
+ *                     daq_call_form() tells which form a call takes;
  *                > 0 = two-pass form with exactly this many CTAs per kernel;
  *                -1 = single-pass plain kernel, one CTA per tile;
  *                -2 = single-pass plain kernel, persistent;

@@ -1010,8 +1010,11 @@ static int make_plan(int n_calo, int n_xtal, int64_t n_samples, int n_fills, con
 // needs enough tiles an SM to gain by the bytes saved.  54 crystals: 51 / 52 at 9.5
 // tiles an SM, 57 / 56 at 11, 63 / 57 at 12.8, 78 / 65 at 16.4, 663 / 496 at 197.
 // Fewer crystals: 53 / 51 at 16.4 (20 crystals), 374 / 328 (12) and 317 / 273 (4) at 197.
+// The line at 14 is one for all counts, drawn by the fewer crystals, which gain least;
+// 54 alone would gain from 11 on.
 // Where the two-pass form would leave the halo out and complete the marks in its scan
-// (post = 64): 37 / 27 at 2, 45 / 42 at 5.7 with 54 crystals, 32 / 33 at 4.1 with 36.
+// (post = 64): 37 / 27 at 2, 45 / 42 at 5.7 with 54 crystals, 32 / 33 at 4.1 with 36;
+// between 36 and 48 crystals nothing was measured, and they keep the line at 14.
 static int phase_min_tiles(const Plan &twopass, int X)  // an SM
 {
     return twopass.halo_free && X >= 48 ? 2 : 14;

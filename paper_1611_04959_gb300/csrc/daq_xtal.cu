@@ -120,8 +120,8 @@ __device__ __forceinline__ void store_q(long long *p, const long long (&v)[8], b
 // 3.03 with lanes on consecutive 16 bytes and 4-byte sample loads.  Groups within a
 // row, taken sample by sample where the pitch is odd, took 1.70 ms for three fills of
 // 24 x 54 x 99,999; these take 0.45.  A sample past its fill's length is not read:
-// eight fills of 24 x 54 x 70,000 cut to 7,000 take 262 us, 465 if it is.  Four CTAs an SM: at five the 64 registers do
-// not suffice (2.22 ms).
+// eight fills of 24 x 54 x 70,000 cut to 7,000 take 262 us, 465 if it is.  Four CTAs an
+// SM: at five the 64 registers do not suffice (2.22 ms).
 // kVec: aligned 16-byte sample loads, of kAhead fills at once (two: 721 us for four
 // fills of 140,000 samples against 731 with one and 748 with four, whose registers
 // cost a CTA); wide: q is 32-byte aligned.  I: the type of rows and places in them, 32
